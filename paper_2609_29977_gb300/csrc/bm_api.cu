@@ -348,7 +348,7 @@ static void prepare_schedule(bm_handle h, const F64View &v, cudaStream_t st) {
     return;
   }
   char kb[320];
-  snprintf(kb, sizeof kb, "fp64-schedule|%.200s|S=%d|N=%d|nb=%d|nr=%d", prop.name, d.S, d.N, d.nb, d.nr);
+  snprintf(kb, sizeof kb, "fp64-schedule-2|%.200s|S=%d|N=%d|nb=%d|nr=%d", prop.name, d.S, d.N, d.nb, d.nr);
   std::vector<int> vals;
   if (tune_cache_lookup(kb, vals) && (int)vals.size() == 1 + (vals.empty() ? 0 : vals[0]) && vals[0] >= 0 &&
       vals[0] <= h->Lc && vals[0] < 32) {

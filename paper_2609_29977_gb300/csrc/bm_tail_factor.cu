@@ -139,7 +139,7 @@ bool tail_factor_tune(const TailView<double> &v, cudaStream_t st, TailSched *bes
       cudaGetLastError();
       return false;
     }
-  const int tmin = nb <= 16 ? 8 : nb <= 32 ? 16 : 32, tmax = nb <= 4 ? 32 : nb <= 16 ? 64 : 128;
+  const int tmin = tail::team_min(nb), tmax = tail::team_max(nb);
   float best_ms[32];
   for (int l = 0; l < 32; ++l) best_ms[l] = 1e30f;
   bool ok = true;

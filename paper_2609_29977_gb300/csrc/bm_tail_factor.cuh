@@ -22,7 +22,7 @@
 #pragma once
 
 #include "bm_root.cuh"
-#include "bm_team.cuh"
+#include "bm_sliced.cuh"
 
 namespace bm {
 namespace tail {
@@ -48,11 +48,54 @@ __device__ __forceinline__ void team_load_t(const Team<TEAM> &tm, T *__restrict_
   }
 }
 
+// The block operations of a task: on the FP64 path the sliced products and
+// the pivots' reciprocals of bm_sliced.cuh for nb >= 12, the plain ones of
+// bm_team.cuh for smaller blocks and for FP32. Whole factor, plain -> sliced:
+// S = 512, N = 128, nb = 24: 6216 -> 3122 us; S = 100, N = 160, nb = 16:
+// 807 -> 438; S = N = 64, nb = 32: 1525 -> 687, nb = 48: 4695 -> 1831, and
+// nb = 12: 153 -> 152, where the line lies: one product of 12 columns costs
+// about as many issue slots as its FP64 FMAs take.
+template <typename T, int NB, int TEAM>
+struct Ops {
+  using Tm = Team<TEAM>;
+  static constexpr bool S = sliced::Use<T, NB>::value;
+  static __device__ __forceinline__ void syrk_sub(const Tm &tm, T *sD, const T *X, const T *Y) {
+    if constexpr (S)
+      sliced::team_syrk_sub<TEAM, NB>(tm, sD, X, Y);
+    else
+      team_syrk_sub<TEAM, NB, T>(tm, sD, X, Y);
+  }
+  static __device__ __forceinline__ int chol(const Tm &tm, T *sA, T *sInv, const sliced::TriTable<NB> &tri) {
+    if constexpr (S)
+      return sliced::team_chol<TEAM, NB>(tm, sA, sInv, tri);
+    else
+      return team_chol<TEAM, NB, T>(tm, sA, sInv);
+  }
+  static __device__ __forceinline__ void store_factor(const Tm &tm, T *g, const T *s, const T *inv) {
+    if constexpr (S)   // team_chol has left the stored form
+      team_copy<TEAM, NB * NB>(tm, g, s);
+    else
+      team_store_factor<TEAM, NB, T>(tm, g, s, inv);
+  }
+  static __device__ __forceinline__ void trsm_lt(const Tm &tm, T *X, int M, T *L, const T *inv) {
+    if constexpr (S)
+      sliced::team_trsm_lt<TEAM, NB>(tm, X, M, L, inv);
+    else
+      team_trsm_lt<TEAM, NB, T>(tm, X, M, L, inv);
+  }
+  static __device__ __forceinline__ void gemm_nt_neg(const Tm &tm, T *out, const T *A, const T *B) {
+    if constexpr (S)
+      sliced::team_gemm_nt_neg<TEAM, NB>(tm, out, A, B);
+    else
+      team_gemm_nt_neg<TEAM, NB, T>(tm, out, A, B);
+  }
+};
+
 // One task of level lvl: the Schur update of position q gathered from its
 // level lvl-1 neighbours and, if q belongs to level lvl, its elimination.
 template <typename T, int NB, int TEAM>
-__device__ __forceinline__ void factor_task(const TailView<T> &v, const Team<TEAM> &tm, T *sD, int s, int q,
-                                            int lvl, bool elim) {
+__device__ __forceinline__ void factor_task(const TailView<T> &v, const Team<TEAM> &tm, T *sD,
+                                            const sliced::TriTable<NB> &tri, int s, int q, int lvl, bool elim) {
   constexpr int NB2 = NB * NB;
   const int N = v.N;
   T *sB = sD + NB2, *sA = sB + NB2, *sInv = sA + NB2;
@@ -75,7 +118,7 @@ __device__ __forceinline__ void factor_task(const TailView<T> &v, const Team<TEA
     if (pl) team_copy<TEAM, NB2>(tm, sB, v.Lr + (sb + (N - pl)) * NB2);
     if (pr) team_copy<TEAM, NB2>(tm, sA, v.Ll + (sb + (N - pr)) * NB2);
     tm.sync();
-    if (pl) team_syrk_sub<TEAM, NB, T>(tm, sD, sB, pr ? sA : nullptr);
+    if (pl) Ops<T, NB, TEAM>::syrk_sub(tm, sD, sB, pr ? sA : nullptr);
     tm.sync();
   }
   if (!elim) {
@@ -101,14 +144,14 @@ __device__ __forceinline__ void factor_task(const TailView<T> &v, const Team<TEA
       team_copy_t<TEAM, NB, T>(tm, sA, v.W + (sb + (N - a)) * NB2);
   }
   tm.sync();
-  const int fail = team_chol<TEAM, NB, T>(tm, sD, sInv);
+  const int fail = Ops<T, NB, TEAM>::chol(tm, sD, sInv, tri);
   if (tm.lane == 0 && fail) report_not_spd(v.status, v.s0 + s, N + 1 - q);
-  team_store_factor<TEAM, NB, T>(tm, v.Ld + (sb + (N - q)) * NB2, sD, sInv);
-  team_trsm_lt<TEAM, NB, T>(tm, sB, hasA ? 2 * NB : NB, sD, sInv);
+  Ops<T, NB, TEAM>::store_factor(tm, v.Ld + (sb + (N - q)) * NB2, sD, sInv);
+  Ops<T, NB, TEAM>::trsm_lt(tm, sB, hasA ? 2 * NB : NB, sD, sInv);
   team_copy<TEAM, NB2>(tm, v.Lr + (sb + (N - q)) * NB2, sB);
   if (hasA) {
     team_copy<TEAM, NB2>(tm, v.Ll + (sb + (N - q)) * NB2, sA);
-    team_gemm_nt_neg<TEAM, NB, T>(tm, v.W + (sb + (N - a)) * NB2, sB, sA);
+    Ops<T, NB, TEAM>::gemm_nt_neg(tm, v.W + (sb + (N - a)) * NB2, sB, sA);
   } else {
     team_zero<TEAM, NB2>(tm, v.Ll + (sb + (N - q)) * NB2);
   }
@@ -125,7 +168,8 @@ __host__ __device__ constexpr size_t x1_bytes(int nr) {
 }
 
 template <typename T, int NB, int TEAM>
-__device__ __forceinline__ void x1_task(const TailView<T> &v, const Team<TEAM> &tm, void *sbuf, int s) {
+__device__ __forceinline__ void x1_task(const TailView<T> &v, const Team<TEAM> &tm, void *sbuf,
+                                        const sliced::TriTable<NB> &tri, int s) {
   constexpr int NB2 = NB * NB;
   const int N = v.N, nr = v.nr, Lc = v.Lc;
   double *sC = (double *)sbuf;
@@ -142,12 +186,12 @@ __device__ __forceinline__ void x1_task(const TailView<T> &v, const Team<TEAM> &
   for (int i = tm.lane; i < nr * NB; i += TEAM) sC[i] = v.C[(size_t)s * nr * NB + i];
   tm.sync();
   if (Lc >= 1) {
-    team_syrk_sub<TEAM, NB, T>(tm, sD, sB, nullptr);
+    Ops<T, NB, TEAM>::syrk_sub(tm, sD, sB, nullptr);
     tm.sync();
   }
-  const int fail = team_chol<TEAM, NB, T>(tm, sD, sInv);
+  const int fail = Ops<T, NB, TEAM>::chol(tm, sD, sInv, tri);
   if (tm.lane == 0 && fail) report_not_spd(v.status, v.s0 + s, 1);
-  team_store_factor<TEAM, NB, T>(tm, v.Ld + sb * NB2, sD, sInv);
+  Ops<T, NB, TEAM>::store_factor(tm, v.Ld + sb * NB2, sD, sInv);
   team_zero<TEAM, NB2>(tm, v.Ll + sb * NB2);
   team_zero<TEAM, NB2>(tm, v.Lr + sb * NB2);
   team_copy<TEAM, NB>(tm, v.invd + sb * NB, sInv);
@@ -186,6 +230,11 @@ __global__ void __launch_bounds__(256) k_factor_level_team(TailView<T> v, int lv
   const int E = level_elims(N, lvl);
   const int G = lvl == 0 ? 0 : ((N - 1) >> (lvl + 1)) + 1;
   const long g = (long)blockIdx.x * tpc + tm.id;
+  __shared__ sliced::TriTable<NB> tri;
+  if (Ops<T, NB, TEAM>::S) {
+    sliced::tri_fill<NB>(tri);
+    __syncthreads();
+  }
   pdl_wait();
   if (g < (long)S * (E + G)) {
     int s, q;
@@ -201,20 +250,33 @@ __global__ void __launch_bounds__(256) k_factor_level_team(TailView<T> v, int lv
       q = j < G - 1 ? (j + 1) << (lvl + 1) : N;
       elim = false;
     }
-    factor_task<T, NB, TEAM>(v, tm, smem + tm.id * TeamSmem<T, NB>::elems, s, q, lvl, elim);
+    factor_task<T, NB, TEAM>(v, tm, smem + tm.id * TeamSmem<T, NB>::elems, tri, s, q, lvl, elim);
   }
   pdl_trigger();
 }
 
+// Teams of the top kernel's CTA. For nb >= 24 two teams of four warps: with
+// four teams of two warps the factor of S = 512, N = 128, nb = 24 takes 3151
+// instead of 3122 us, and four of four spill (128 registers).
+template <typename T, int NB>
+constexpr int top_teams() {
+  return NB <= 16 ? 4 : 2;
+}
+
 // Top levels lvl0..Lc-1 and x_1 of one tail per CTA.
 template <typename T, int NB, int TEAM>
-__global__ void __launch_bounds__(512) k_factor_top(TailView<T> v, int lvl0) {
+__global__ void __launch_bounds__(TEAM * top_teams<T, NB>()) k_factor_top(TailView<T> v, int lvl0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *smem = (T *)smem_raw;
   const Team<TEAM> tm;
   const int tpc = blockDim.x / TEAM;
   const int N = v.N, s = blockIdx.x;
   constexpr int per = TeamSmem<T, NB>::elems;
+  __shared__ sliced::TriTable<NB> tri;
+  if (Ops<T, NB, TEAM>::S) {
+    sliced::tri_fill<NB>(tri);
+    __syncthreads();
+  }
   pdl_wait();
   for (int lvl = lvl0; lvl < v.Lc; ++lvl) {
     const int E = level_elims(N, lvl);
@@ -222,11 +284,11 @@ __global__ void __launch_bounds__(512) k_factor_top(TailView<T> v, int lvl0) {
     for (int t = tm.id; t < E + G; t += tpc) {
       const bool elim = t < E;
       const int q = elim ? (2 * t + 1) << lvl : (t - E < G - 1 ? (t - E + 1) << (lvl + 1) : N);
-      factor_task<T, NB, TEAM>(v, tm, smem + tm.id * per, s, q, lvl, elim);
+      factor_task<T, NB, TEAM>(v, tm, smem + tm.id * per, tri, s, q, lvl, elim);
     }
     __syncthreads();
   }
-  if (tm.id == 0) x1_task<T, NB, TEAM>(v, tm, smem_raw, s);
+  if (tm.id == 0) x1_task<T, NB, TEAM>(v, tm, smem_raw, tri, s);
   if constexpr (sizeof(T) == sizeof(double)) {
     if (v.LR) {
       // the last tail to finish its U_i does the root step (Alg. 1 steps 4-5)
@@ -246,7 +308,7 @@ __global__ void __launch_bounds__(512) k_factor_top(TailView<T> v, int lvl0) {
 }
 
 // Team sizes compiled for each block size, and the team of the top kernel.
-constexpr int team_min(int nb) { return nb <= 16 ? 8 : nb <= 32 ? 16 : 32; }
+constexpr int team_min(int nb) { return nb <= 8 ? 8 : 32; }
 constexpr int team_max(int nb) { return nb <= 4 ? 32 : nb <= 16 ? 64 : 128; }
 constexpr int team_top(int nb) { return nb <= 8 ? 32 : nb <= 16 ? 64 : 128; }
 
@@ -277,8 +339,7 @@ template <typename T, int NB, int TEAM>
 void launch_top(const TailView<T> &v, int lvl0, cudaStream_t st) {
   const size_t per = TeamSmem<T, NB>::bytes;
   const size_t x1b = x1_bytes<T, NB>(v.nr);
-  int tpc = TEAM >= 128 ? 4 : 512 / TEAM > 4 ? 4 : 512 / TEAM;
-  while (tpc > 1 && per * tpc > 200 * 1024) tpc >>= 1;
+  constexpr int tpc = top_teams<T, NB>();
   size_t smem = per * tpc > x1b ? per * tpc : x1b;
   const size_t rootb = ((size_t)v.nr * v.nr + v.nr) * sizeof(double);
   if (v.LR && rootb > smem) smem = rootb;
@@ -289,9 +350,11 @@ template <typename T, int NB, int TEAM>
 cudaError_t prepare_one() {
   cudaError_t e = cudaFuncSetAttribute(k_factor_level_team<T, NB, TEAM>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_factor_top<T, NB, TEAM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              210 * 1024);
+  if constexpr (TEAM == team_top(NB)) {
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_factor_top<T, NB, TEAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024);
+  }
+  return e;
 }
 
 template <typename T, int NB, int TEAM>

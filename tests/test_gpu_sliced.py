@@ -1,0 +1,120 @@
+"""FP64 tail factor with sliced tensor-core products (nb >= 12,
+csrc/bm_sliced.cuh): its backward error in extended precision, and the
+properties that the digits must not break.
+
+Bound of the backward error: the blocks of L satisfy, entry by entry,
+|K - L L^T|_ij <= gamma sqrt(K_ii K_jj) for a backward-stable Cholesky with
+gamma = (m + 1) u, u = 2^-53 and m the longest sum behind an entry (Demmel,
+"On floating point errors in Cholesky", 1989). An entry of a chain position
+gathers two nb-term products per level and the nb terms of its own block:
+m = nb (2 levels + 1). The same bound holds for FP64 FMAs; the sliced
+products, with one rounding per product, have to meet it as well.
+"""
+import numpy as np
+import pytest
+import torch
+
+import bmgen
+
+pytestmark = pytest.mark.gpu
+
+# every compiled block size from 12 up; N at powers of two and beside them
+SHAPES = [(2, 9, 12, 4), (1, 17, 16, 16), (2, 6, 16, 5), (2, 13, 24, 8), (1, 2, 24, 8), (1, 8, 32, 11), (1, 5, 48, 16)]
+
+
+def _bm():
+    import paper_2609_29977_gb300 as bm
+    return bm
+
+
+def _gen(S, N, nb, nr, seed=3):
+    return bmgen.generate(bmgen.Workload("t", S, N, nb, nr, barrier=(-4.0, 4.0), shared_A=True), seed=seed)
+
+
+def _run(d, flags=0):
+    bm = _bm()
+    g = {k: (v.cuda() if isinstance(v, torch.Tensor) else v) for k, v in d.items()}
+    s = bm.BranchKKTSolver(d["S"], d["N"], d["nb"], d["nr"], flags=flags)
+    s.factor(g["D"], g["E"], g["C"], g["R"])
+    x = s.solve(g["r"]).cpu().numpy()
+    fac = {k: v.cpu().numpy() for k, v in s.export_factor().items()}
+    info = s.query()
+    s.close()
+    return x, fac, info
+
+
+@pytest.mark.parametrize("S,N,nb,nr", SHAPES)
+def test_backward_error_of_the_tail_factor(S, N, nb, nr):
+    d = _gen(S, N, nb, nr)
+    _, fac, info = _run(d)
+    assert info["status"] == 0
+    D, E = d["D"].numpy(), d["E"].numpy()
+    levels = (N - 1).bit_length()
+    gamma = (nb * (2 * levels + 1) + 1) * 2.0 ** -53
+    for s in range(S):
+        # rows of the tail by chain position p = N + 1 - k; column p of L has
+        # the blocks (p, p), (left neighbour, p), (right neighbour, p)
+        n = N * nb
+        K = np.zeros((n, n), dtype=np.longdouble)
+        L = np.zeros((n, n), dtype=np.longdouble)
+        at = lambda p: slice((p - 1) * nb, p * nb)  # noqa: E731
+        for p in range(1, N + 1):
+            k = N - p                                # natural stage index
+            K[at(p), at(p)] = np.tril(D[s, k]) + np.tril(D[s, k], -1).T
+            if p < N:                                # (stage k+1, stage k) = E[k-1]
+                K[at(p), at(p + 1)] = E[s, k - 1]
+                K[at(p + 1), at(p)] = E[s, k - 1].T
+            L[at(p), at(p)] = np.tril(fac["Ld"][s, k])
+            if p < N:
+                h = p & -p
+                right = p + h if p + h <= N - 1 else N
+                L[at(right), at(p)] = fac["Lr"][s, k]
+                if p > h:
+                    L[at(p - h), at(p)] = fac["Ll"][s, k]
+        err = np.abs(K - L @ L.T)
+        scale = np.sqrt(np.outer(np.diag(K), np.diag(K)))
+        assert float((err / scale).max()) <= gamma, float((err / scale).max()) / gamma
+
+
+@pytest.mark.parametrize("S,N,nb,nr", [(2, 13, 24, 8), (2, 9, 12, 4)])
+def test_scaling_by_powers_of_two_is_exact(S, N, nb, nr):
+    """K scaled by an even power of two scales L and x exactly: the digits
+    are taken relative to each row's exponent."""
+    d = _gen(S, N, nb, nr)
+    x, fac, _ = _run(d)
+    for k in (600, -600):
+        f = 2.0 ** k
+        e = dict(d, D=d["D"] * f, E=d["E"] * f, C=d["C"] * f, R=d["R"] * f)
+        xs, fs, info = _run(e)
+        assert info["status"] == 0
+        assert np.array_equal(xs * f, x)
+        assert np.array_equal(fs["Lr"] * 2.0 ** (-k // 2), fac["Lr"])
+
+
+@pytest.mark.parametrize("S,N,nb,nr", [(3, 37, 24, 8), (3, 37, 16, 4), (2, 11, 48, 16)])
+def test_team_sizes_and_top_levels_give_the_same_bits(S, N, nb, nr, tmp_path, monkeypatch):
+    """Schedules of the cache file, of every compiled team size and two top
+    levels, against the default rule."""
+    import json
+    bm = _bm()
+    d = _gen(S, N, nb, nr)
+    ref, fac, _ = _run(d, flags=bm.BM_FLAG_NO_TUNE)
+    monkeypatch.setenv("BM_AUTOTUNE_CACHE", str(tmp_path / "tune.json"))
+    _run(d)                                          # writes the entry
+    path = tmp_path / "tune.json"
+    key = next(k for k in json.loads(path.read_text()) if "fp64-schedule" in k)
+    for team in (32, 64, 128):
+        for top in (2, 3):
+            path.write_text(json.dumps({key: [top] + [team] * top}))
+            x, f, _ = _run(d)
+            assert np.array_equal(x, ref) and all(np.array_equal(f[k], fac[k]) for k in fac), (team, top)
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("nb", [12, 24])
+def test_non_finite_coupling_is_reported(nb, bad):
+    d = _gen(2, 9, nb, 4)
+    d["E"] = d["E"].clone()
+    d["E"][1, 3, nb - 1, 2] = bad
+    _, _, info = _run(d)
+    assert info["name"] == "BM_ERR_NOT_SPD" and info["fail_scenario"] == 1
