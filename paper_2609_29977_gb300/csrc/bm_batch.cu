@@ -613,7 +613,7 @@ extern "C" bm_status bm_batch_analyze(const bm_desc *descs, int count, void *str
   char kb[256];
   long tot_stages = 0;
   for (int b = 0; b < count; ++b) tot_stages += (long)descs[b].S * descs[b].N;
-  snprintf(kb, sizeof kb, "%.200s|n=%d|stages~2^%d|nb=", prop.name, count, 63 - __builtin_clzll((unsigned long long)tot_stages | 1));
+  snprintf(kb, sizeof kb, "%.200s|rows-2|n=%d|stages~2^%d|nb=", prop.name, count, 63 - __builtin_clzll((unsigned long long)tot_stages | 1));
   h->key = kb;
   for (int nb : nbs) h->key += std::to_string(nb) + ",";
   *out = h;

@@ -21,8 +21,14 @@ namespace rows {
 template <int NB>
 struct Cfg {
   static constexpr int TS = NB <= 4 ? 4 : NB <= 8 ? 8 : NB <= 16 ? 16 : 32;
-  static constexpr int LD = NB + 1;   // padded row stride of staged blocks (no bank conflicts)
-  static constexpr int SM = NB * LD;  // staged block size in elements
+  // Blocks whose rows are groups of four floats move through shared memory
+  // (factor_task_staged); the others (nb = 2, 3, 6) keep one staged block.
+  static constexpr bool STAGED = NB % 4 == 0;
+  // row stride of staged blocks without bank conflicts: an odd number of
+  // 16-byte groups (rows read and written four floats at a time), or NB + 1
+  static constexpr int LD = STAGED ? (NB / 4 % 2 ? NB : NB + 4) : NB + 1;
+  static constexpr int BLK = NB * LD;               // one staged block
+  static constexpr int SM = STAGED ? 4 * BLK : BLK; // per team
 };
 
 template <typename T>
@@ -162,13 +168,234 @@ __device__ __forceinline__ int chol_trsm_rows(T (&d)[NB], T (&b)[NB], T (&a)[NB]
   return fail;
 }
 
-// One task of level lvl with register-resident rows.
+// 16-byte asynchronous copy, global to shared memory through L2.
+__device__ __forceinline__ void cp_async16(void *s, const void *g) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(s)), "l"(g)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// An NB x NB float block, global (contiguous) <-> shared memory (row stride
+// LD), 16 bytes per access and contiguous over the team.
+template <int NB, int TS, int LD = Cfg<NB>::LD>
+__device__ __forceinline__ void block_in(float *__restrict__ s, const float *__restrict__ g, int lane) {
+#pragma unroll
+  for (int e = lane; e < NB * NB / 4; e += TS) {
+    const int r = 4 * e / NB, c = 4 * e - r * NB;
+    cp_async16(s + r * LD + c, g + 4 * e);
+  }
+}
+template <int NB, int TS, int LD = Cfg<NB>::LD>
+__device__ __forceinline__ void block_out(float *__restrict__ g, const float *__restrict__ s, int lane) {
+#pragma unroll
+  for (int e = lane; e < NB * NB / 4; e += TS) {
+    const int r = 4 * e / NB, c = 4 * e - r * NB;
+    reinterpret_cast<float4 *>(g)[e] = *reinterpret_cast<const float4 *>(s + r * LD + c);
+  }
+}
+// An FP64 input block, rounded to FP32, into shared memory: two doubles per
+// load, contiguous over the team, all loads before the first conversion (the
+// hardware rounding, see load_to_t). LOWER: only pairs that reach the lower triangle.
+template <int NB, int TS, bool LOWER, int LD = Cfg<NB>::LD>
+__device__ __forceinline__ void block_in_d(float *__restrict__ s, const double *__restrict__ g, int lane) {
+  // 9 loads in flight per lane (all of a 24 x 24 block, half of a 48 x 48 one)
+  constexpr int Q = NB * NB / 2, M = (Q + TS - 1) / TS, CH = M < 9 ? M : 9;
+#pragma unroll
+  for (int t0 = 0; t0 < M; t0 += CH) {
+    double2 v[CH];
+#pragma unroll
+    for (int t = 0; t < CH; ++t) {
+      const int e = lane + (t0 + t) * TS, r = 2 * e / NB, c = 2 * e - r * NB;
+      if (e < Q && (!LOWER || c <= r)) v[t] = reinterpret_cast<const double2 *>(g)[e];
+    }
+#pragma unroll
+    for (int t = 0; t < CH; ++t) {
+      const int e = lane + (t0 + t) * TS, r = 2 * e / NB, c = 2 * e - r * NB;
+      if (e < Q && (!LOWER || c <= r))
+        *reinterpret_cast<float2 *>(s + r * LD + c) =
+            make_float2(__double2float_rn(v[t].x), __double2float_rn(v[t].y));
+    }
+  }
+}
+// A row of a staged block <-> registers.
+template <int NB>
+__device__ __forceinline__ void row_in(float (&d)[NB], const float *__restrict__ row) {
+#pragma unroll
+  for (int g = 0; g < NB / 4; ++g) {
+    const float4 v = reinterpret_cast<const float4 *>(row)[g];
+    d[4 * g] = v.x;
+    d[4 * g + 1] = v.y;
+    d[4 * g + 2] = v.z;
+    d[4 * g + 3] = v.w;
+  }
+}
+template <int NB>
+__device__ __forceinline__ void row_out(float *__restrict__ row, const float (&d)[NB]) {
+#pragma unroll
+  for (int g = 0; g < NB / 4; ++g)
+    reinterpret_cast<float4 *>(row)[g] = make_float4(d[4 * g], d[4 * g + 1], d[4 * g + 2], d[4 * g + 3]);
+}
+// sum_k a[k] row[k], k in increasing order (row staged, read by all lanes).
+template <int NB>
+__device__ __forceinline__ float row_dot(const float (&a)[NB], const float *__restrict__ row) {
+  float acc = 0.0f;
+#pragma unroll
+  for (int g = 0; g < NB / 4; ++g) {
+    const float4 v = reinterpret_cast<const float4 *>(row)[g];
+    acc = fmaf(a[4 * g], v.x, acc);
+    acc = fmaf(a[4 * g + 1], v.y, acc);
+    acc = fmaf(a[4 * g + 2], v.z, acc);
+    acc = fmaf(a[4 * g + 3], v.w, acc);
+  }
+  return acc;
+}
+
+// One task of level lvl with register-resident rows, every block moved
+// between global and shared memory contiguously (16 bytes per lane) and
+// between shared memory and the lanes' rows without bank conflicts. With a
+// lane per row, rows loaded and stored straight from global memory put each
+// lane of an access on a line of its own: for nb = 24 about 3500 L1 tag
+// cycles per task of level 0, which took most of the level's time. The
+// float blocks of a task (D~, both neighbours' couplings, the fill) are
+// requested together, before anything waits for one of them.
+// S = 512, N = 128, nb = 24: level 0 405 -> 252 us, level 1 321 -> 214,
+// FP32+IR factor and solve 4304 -> 3919 us; S = N = 64, nb = 12: 288 -> 277.
+// What bounds level 0 now is the conversion of
+// the FP64 inputs (FP64 pipe 44%) and the columns' shuffle chains.
+// The arithmetic and its order are those of factor_task_plain.
 // FUSED: the Cholesky and the coupling solves in one column loop
 // (chol_trsm_rows; the grid-wide level kernel) or one after the other (the
 // per-tail top kernel and the batched form, whose register budget the
 // fused loop would exceed). Both give the same bits.
+// buf: Cfg<NB>::SM floats per team, 16-byte aligned.
+template <int NB, bool FUSED>
+__device__ __forceinline__ void factor_task_staged(const TailView<float> &v, float *buf, int lane, unsigned mask,
+                                                   int s, int q, int lvl, bool elim) {
+  constexpr int TS = Cfg<NB>::TS, NB2 = NB * NB, LD = Cfg<NB>::LD, BLK = Cfg<NB>::BLK;
+  float *b0 = buf, *b1 = buf + BLK, *b2 = b1 + BLK, *b3 = b2 + BLK;
+  const int N = v.N;
+  const size_t sb = (size_t)s * N;
+  const int i = lane;
+  const bool act = i < NB;
+  const int ir = act ? i : 0;
+  int pl = 0, pr = 0;
+  if (lvl >= 1) {
+    const int h = 1 << (lvl - 1);
+    if (q < N) {
+      pl = q - h;
+      if (q + h <= N - 1) pr = q + h;
+    } else {
+      const int m = ((N - 1) >> (lvl - 1)) << (lvl - 1);
+      if (ctz32(m) == lvl - 1) pl = m;
+    }
+  }
+  const int hh = 1 << lvl;
+  const bool hasA = q > hh;
+  const int a = q - hh;
+  const bool inputB = lvl == 0 || q == N - 1;   // M_{b,q} is an input block (E^T)
+  if (lvl >= 2) block_in<NB, TS>(b0, v.Dt + (sb + (N - q)) * NB2, lane);
+  if (pl) block_in<NB, TS>(b1, v.Lr + (sb + (N - pl)) * NB2, lane);
+  if (pr) block_in<NB, TS>(b2, v.Ll + (sb + (N - pr)) * NB2, lane);
+  if (elim && !inputB) block_in<NB, TS>(b3, v.W + (sb + (N - q)) * NB2, lane);
+  if (lvl <= 1) block_in_d<NB, TS, true>(b0, v.D + (sb + (N - q)) * NB2, lane);
+  if (lvl == 0 && hasA) block_in_d<NB, TS, false>(b2, v.E + ((size_t)s * (N - 1) + (N - q)) * NB2, lane);
+  cp_async_wait();
+  __syncwarp(mask);
+  float d[NB];
+  if (lvl <= 1) {
+#pragma unroll
+    for (int j = 0; j < NB; ++j) d[j] = j <= ir ? b0[ir * LD + j] : b0[j * LD + ir];
+  } else {
+    row_in<NB>(d, b0 + ir * LD);
+  }
+  if (pl) {
+    float x[NB];
+    row_in<NB>(x, b1 + ir * LD);
+#pragma unroll
+    for (int j = 0; j < NB; ++j) d[j] -= row_dot<NB>(x, b1 + j * LD);
+  }
+  if (pr) {
+    float x[NB];
+    row_in<NB>(x, b2 + ir * LD);
+#pragma unroll
+    for (int j = 0; j < NB; ++j) d[j] -= row_dot<NB>(x, b2 + j * LD);
+  }
+  __syncwarp(mask);   // the staged inputs have been read
+  if (!elim) {
+    if (act) row_out<NB>(b0 + i * LD, d);
+    __syncwarp(mask);
+    block_out<NB, TS>(v.Dt + (sb + (N - q)) * NB2, b0, lane);
+    __syncwarp(mask);
+    return;
+  }
+  // couplings: rows i of M_{b,q} and M_{a,q}
+  float b[NB], av[NB];
+  if (inputB) {
+    const double *Eb = v.E + ((size_t)s * (N - 1) + (N - q - 1)) * NB2;   // M_{b,q} = E^T: contiguous over the lanes
+    load_to_t<float, NB>(b, [&](int k) { return Eb[k * NB + ir]; });
+  } else {
+    row_in<NB>(b, b3 + ir * LD);
+  }
+  if (hasA) {
+    if (lvl == 0) {
+      row_in<NB>(av, b2 + ir * LD);
+    } else {
+      const float *Wa = v.W + (sb + (N - a)) * NB2;   // M_{a,q} = W[a]^T: contiguous over the lanes
+#pragma unroll
+      for (int k = 0; k < NB; ++k) av[k] = Wa[k * NB + ir];
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < NB; ++k) av[k] = 0.0f;
+  }
+  float rinv = 1.0f;
+  int fail;
+  if constexpr (FUSED) {
+    // one instantiation for both cases: without a left neighbour av is zero
+    // and stays +0 through the updates
+    fail = chol_trsm_rows<float, NB, TS, true>(d, b, av, rinv, mask, i);
+  } else {
+    fail = chol_rows<float, NB, TS>(d, rinv, mask, i);
+    if (hasA)
+      trsm_rows<float, NB, TS, true>(b, av, d, rinv, mask);
+    else
+      trsm_rows<float, NB, TS, false>(b, av, d, rinv, mask);
+  }
+  if (i == 0 && fail) report_not_spd(v.status, s, N + 1 - q);
+  if (act) {
+#pragma unroll
+    for (int j = 0; j < NB; ++j)
+      if (j > i) d[j] = 0.0f;
+    row_out<NB>(b0 + i * LD, d);
+    row_out<NB>(b1 + i * LD, b);
+    row_out<NB>(b2 + i * LD, av);
+    v.invd[(sb + (N - q)) * NB + i] = rinv;
+  }
+  __syncwarp(mask);
+  block_out<NB, TS>(v.Ld + (sb + (N - q)) * NB2, b0, lane);
+  block_out<NB, TS>(v.Lr + (sb + (N - q)) * NB2, b1, lane);
+  block_out<NB, TS>(v.Ll + (sb + (N - q)) * NB2, b2, lane);
+  if (hasA) {
+    // fill M_{b,a} = -L_{b,q} L_{a,q}^T (rows of L_{a,q} in b2)
+    if (act) {
+#pragma unroll
+      for (int g = 0; g < NB / 4; ++g) {
+        float w[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) w[e] = -row_dot<NB>(b, b2 + (4 * g + e) * LD);
+        reinterpret_cast<float4 *>(b3 + i * LD)[g] = make_float4(w[0], w[1], w[2], w[3]);
+      }
+    }
+    __syncwarp(mask);
+    block_out<NB, TS>(v.W + (sb + (N - a)) * NB2, b3, lane);
+  }
+  __syncwarp(mask);
+}
+
+// One task of level lvl with register-resident rows loaded and stored
+// straight from global memory (block sizes without groups of four).
 template <typename T, int NB, bool FUSED = false>
-__device__ __forceinline__ void factor_task_rows(const TailView<T> &v, T *sX, int lane, unsigned mask, int s, int q,
+__device__ __forceinline__ void factor_task_plain(const TailView<T> &v, T *sX, int lane, unsigned mask, int s, int q,
                                                  int lvl, bool elim) {
   constexpr int TS = Cfg<NB>::TS, NB2 = NB * NB;
   const int N = v.N;
@@ -290,6 +517,15 @@ __device__ __forceinline__ void factor_task_rows(const TailView<T> &v, T *sX, in
   }
 }
 
+template <typename T, int NB, bool FUSED = false>
+__device__ __forceinline__ void factor_task_rows(const TailView<T> &v, T *sX, int lane, unsigned mask, int s, int q,
+                                                 int lvl, bool elim) {
+  if constexpr (Cfg<NB>::STAGED)
+    factor_task_staged<NB, FUSED>(v, sX, lane, mask, s, q, lvl, elim);
+  else
+    factor_task_plain<T, NB, FUSED>(v, sX, lane, mask, s, q, lvl, elim);
+}
+
 // x_1 of tail s: last update and L_{i,1} with register rows, then F_{i,1} =
 // C_{i,1} L_{i,1}^{-T} and U_i = F F^T in FP64. sbuf: nr*NB doubles followed
 // by NB*NB + NB values of type T.
@@ -367,7 +603,7 @@ __device__ __forceinline__ void x1_task_rows(const TailView<T> &v, void *sbuf, i
 
 template <typename T, int NB>
 __host__ __device__ constexpr size_t x1_rows_bytes(int nr) {
-  return (size_t)nr * NB * sizeof(double) + (NB * (NB + 1) + NB) * sizeof(T);
+  return (size_t)nr * NB * sizeof(double) + (NB * Cfg<NB>::LD + NB) * sizeof(T);
 }
 
 }  // namespace rows
@@ -435,7 +671,7 @@ __global__ void __launch_bounds__(128) k_top_rows(TailView<T> v, int lvl0) {
 
 template <typename T, int NB>
 cudaError_t prepare_rows() {
-  cudaError_t e = cudaFuncSetAttribute(k_level_rows<T, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+  cudaError_t e = cudaFuncSetAttribute(k_level_rows<T, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_top_rows<T, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
 }

@@ -1,6 +1,7 @@
-"""FP64 tail factor with sliced tensor-core products (nb >= 12,
-csrc/bm_sliced.cuh): its backward error in extended precision, and the
-properties that the digits must not break.
+"""Backward error of the tail factor in extended precision: FP64 with sliced
+tensor-core products (nb >= 12, csrc/bm_sliced.cuh), and the FP32 tails of the
+mixed path (csrc/bm_tail_rows.cuh), whose blocks move through shared memory;
+and the properties that the digits must not break.
 
 Bound of the backward error: the blocks of L satisfy, entry by entry,
 |K - L L^T|_ij <= gamma sqrt(K_ii K_jj) for a backward-stable Cholesky with
@@ -8,7 +9,8 @@ gamma = (m + 1) u, u = 2^-53 and m the longest sum behind an entry (Demmel,
 "On floating point errors in Cholesky", 1989). An entry of a chain position
 gathers two nb-term products per level and the nb terms of its own block:
 m = nb (2 levels + 1). The same bound holds for FP64 FMAs; the sliced
-products, with one rounding per product, have to meet it as well.
+products, with one rounding per product, have to meet it as well. FP32 tails:
+u = 2^-24, and one more rounding for the inputs (m + 2).
 """
 import numpy as np
 import pytest
@@ -31,10 +33,10 @@ def _gen(S, N, nb, nr, seed=3):
     return bmgen.generate(bmgen.Workload("t", S, N, nb, nr, barrier=(-4.0, 4.0), shared_A=True), seed=seed)
 
 
-def _run(d, flags=0):
+def _run(d, flags=0, precision=0):
     bm = _bm()
     g = {k: (v.cuda() if isinstance(v, torch.Tensor) else v) for k, v in d.items()}
-    s = bm.BranchKKTSolver(d["S"], d["N"], d["nb"], d["nr"], flags=flags)
+    s = bm.BranchKKTSolver(d["S"], d["N"], d["nb"], d["nr"], precision=precision, flags=flags)
     s.factor(g["D"], g["E"], g["C"], g["R"])
     x = s.solve(g["r"]).cpu().numpy()
     fac = {k: v.cpu().numpy() for k, v in s.export_factor().items()}
@@ -43,14 +45,11 @@ def _run(d, flags=0):
     return x, fac, info
 
 
-@pytest.mark.parametrize("S,N,nb,nr", SHAPES)
-def test_backward_error_of_the_tail_factor(S, N, nb, nr):
-    d = _gen(S, N, nb, nr)
-    _, fac, info = _run(d)
-    assert info["status"] == 0
+def _check_backward_error(d, fac, terms, u):
+    S, N, nb = d["S"], d["N"], d["nb"]
     D, E = d["D"].numpy(), d["E"].numpy()
     levels = (N - 1).bit_length()
-    gamma = (nb * (2 * levels + 1) + 1) * 2.0 ** -53
+    gamma = (nb * (2 * levels + 1) + terms) * u
     for s in range(S):
         # rows of the tail by chain position p = N + 1 - k; column p of L has
         # the blocks (p, p), (left neighbour, p), (right neighbour, p)
@@ -74,6 +73,25 @@ def test_backward_error_of_the_tail_factor(S, N, nb, nr):
         err = np.abs(K - L @ L.T)
         scale = np.sqrt(np.outer(np.diag(K), np.diag(K)))
         assert float((err / scale).max()) <= gamma, float((err / scale).max()) / gamma
+
+
+@pytest.mark.parametrize("S,N,nb,nr", SHAPES)
+def test_backward_error_of_the_tail_factor(S, N, nb, nr):
+    d = _gen(S, N, nb, nr)
+    _, fac, info = _run(d)
+    assert info["status"] == 0
+    _check_backward_error(d, fac, 1, 2.0 ** -53)
+
+
+# every block size of the staged FP32 tasks, the plain ones (3, 6) beside them
+@pytest.mark.parametrize("S,N,nb,nr", [(3, 9, 3, 2), (9, 16, 4, 2), (2, 12, 6, 2), (5, 17, 8, 3), (3, 13, 12, 4),
+                                       (3, 7, 16, 5), (2, 21, 24, 8), (1, 6, 32, 11), (2, 11, 48, 16), (1, 2, 48, 3)])
+def test_backward_error_of_the_fp32_tail_factor(S, N, nb, nr):
+    bm = _bm()
+    d = _gen(S, N, nb, nr)
+    d["D"], d["E"] = d["D"].float().double(), d["E"].float().double()   # the factor's own inputs
+    _, fac, _ = _run(d, precision=bm.BM_PREC_FP32_IR)
+    _check_backward_error(d, fac, 2, 2.0 ** -24)
 
 
 @pytest.mark.parametrize("S,N,nb,nr", [(2, 13, 24, 8), (2, 9, 12, 4)])
