@@ -38,7 +38,7 @@
 #include <vector>
 
 #include "bm_batch.cuh"
-#include "bm_tail_rows.cuh"
+#include "bm_tail_wide.cuh"
 
 namespace bm {
 bool tune_cache_lookup(const std::string &key, std::vector<int> &vals);
@@ -158,7 +158,7 @@ __device__ __forceinline__ const BSeg &find_seg(const BClass &c, long idx) {
 }
 
 // Worker loop of one team over the queue of class c: register-row tasks,
-// one warp or less per task for block sizes <= 32, two warps (named barrier
+// one warp or less per task for block sizes <= 32, three warps (named barrier
 // per team) for larger blocks.
 template <int NB>
 __device__ void class_worker(const BClass &c, const BInst *inst, const double *const *Dp, const double *const *Ep,
@@ -167,7 +167,7 @@ __device__ void class_worker(const BClass &c, const BInst *inst, const double *c
   constexpr bool WIDE = NB > 32;
   constexpr int NBn = WIDE ? 32 : NB;        // narrow instantiation (unused when WIDE)
   constexpr int NBw = WIDE ? NB : 48;        // wide instantiation (unused when narrow)
-  constexpr int TS = WIDE ? 64 : rows::Cfg<NBn>::TS;
+  constexpr int TS = WIDE ? rows::WCfg<NBw>::TS : rows::Cfg<NBn>::TS;
   const int team = threadIdx.x / TS, lane = threadIdx.x % TS;
   const unsigned mask =
       TS >= 32 ? 0xffffffffu : (((1u << (TS & 31)) - 1u) << ((threadIdx.x & 31) / TS * TS));
@@ -215,7 +215,7 @@ __device__ void class_worker(const BClass &c, const BInst *inst, const double *c
         team_sync();
       }
       if (WIDE)
-        rows::factor_task_rows_w<float, NBw>(v, (float *)tsm, lane, bar, s, q, lvl, elim);
+        rows::factor_task_w<NBw>(v, (float *)tsm, lane, bar, s, q, lvl, elim);
       else
         rows::factor_task_rows<float, NBn>(v, (float *)tsm, lane, mask, s, q, lvl, elim);
       team_sync();
@@ -227,7 +227,7 @@ __device__ void class_worker(const BClass &c, const BInst *inst, const double *c
         team_sync();
       }
       if (WIDE)
-        rows::x1_task_rows_w<float, NBw>(v, tsm, lane, bar, s);
+        rows::x1_task_w<NBw>(v, tsm, lane, bar, s);
       else
         rows::x1_task_rows<float, NBn>(v, tsm, lane, mask, s);
       team_sync();
@@ -268,7 +268,7 @@ __global__ void k_batch_prep(BInst *inst, int ninst, BClass *cls, int ncls, cons
 // holding one class's code, instead of one launch whose CTAs visit every
 // class (and whose SMs then ran the task bodies of all block sizes at once).
 template <int NB>
-__global__ void __launch_bounds__(256) k_batch_factor_nb(const BClass *cls, int c, BInst *inst,
+__global__ void __launch_bounds__(NB > 32 ? 384 : 256) k_batch_factor_nb(const BClass *cls, int c, BInst *inst,
                                                          const double *const *Dp, const double *const *Ep,
                                                          const double *const *Cp, const double *const *Rp,
                                                          unsigned long long limit) {
@@ -287,11 +287,16 @@ int team_bytes_for(int nr) {
     return (int)align_up(a > b ? a : b, 16);
   }
   const size_t a = (size_t)rows::WCfg<(NB > 32 ? NB : 48)>::ELEMS * sizeof(float);
-  const size_t b = rows::x1_rows_w_bytes<float, (NB > 32 ? NB : 48)>(nr);
+  const size_t b = rows::x1_w_bytes<(NB > 32 ? NB : 48)>(nr);
   return (int)align_up(a > b ? a : b, 16);
 }
 
-int team_width(int nb) { return nb <= 4 ? 4 : nb <= 8 ? 8 : nb <= 16 ? 16 : nb <= 32 ? 32 : 64; }
+int team_width(int nb) { return nb <= 4 ? 4 : nb <= 8 ? 8 : nb <= 16 ? 16 : nb <= 32 ? 32 : 96; }
+// Teams per CTA, and the CTA's threads, of a class for the tuned thread
+// count (64, 128 or 256): the three-warp teams of nb = 48 take 96 threads for
+// every 64.
+int class_teams(int threads, int nb) { return nb <= 32 ? threads / team_width(nb) : threads / 64; }
+int class_threads(int threads, int nb) { return nb <= 32 ? threads : class_teams(threads, nb) * team_width(nb); }
 
 int batch_team_bytes(int nb, int nr) {
   switch (nb) {
@@ -407,8 +412,7 @@ extern "C" size_t bm_batch_workspace_bytes(const bm_desc *descs, int count) {
 static size_t smem_for(const bm_batch_s *h, int threads) {
   size_t best = 0;
   for (int c = 0; c < h->ncls; ++c) {
-    const int tw = team_width(h->cls_nb[c]);
-    const size_t need = (size_t)(threads / tw) * h->cls_team_bytes[c];
+    const size_t need = (size_t)class_teams(threads, h->cls_nb[c]) * h->cls_team_bytes[c];
     best = need > best ? need : best;
   }
   return best;
@@ -417,16 +421,17 @@ static size_t smem_for(const bm_batch_s *h, int threads) {
 static void launch_class(bm_batch_s *h, int c, const double *const *D, const double *const *E,
                          const double *const *C, const double *const *R, cudaStream_t st, bool pdl) {
   const unsigned grid = (unsigned)(h->sms * h->ctas_per_sm);
-  const size_t smem = (size_t)(h->threads / team_width(h->cls_nb[c])) * h->cls_team_bytes[c];
+  const unsigned threads = (unsigned)class_threads(h->threads, h->cls_nb[c]);
+  const size_t smem = (size_t)class_teams(h->threads, h->cls_nb[c]) * h->cls_team_bytes[c];
   const unsigned long long limit = 4000000000ull;   // about 2 s of SM clock
   switch (h->cls_nb[c]) {
 #define X(n)                                                                                                    \
   case n:                                                                                                       \
     if (pdl)                                                                                                    \
-      launch_pdl(k_batch_factor_nb<n>, grid, (unsigned)h->threads, smem, st, (const BClass *)h->d_cls, c,      \
+      launch_pdl(k_batch_factor_nb<n>, grid, threads, smem, st, (const BClass *)h->d_cls, c,                   \
                  h->d_inst, D, E, C, R, limit);                                                                 \
     else                                                                                                        \
-      k_batch_factor_nb<n><<<grid, h->threads, smem, st>>>(h->d_cls, c, h->d_inst, D, E, C, R, limit);        \
+      k_batch_factor_nb<n><<<grid, threads, smem, st>>>(h->d_cls, c, h->d_inst, D, E, C, R, limit);        \
     break;
     BM_BATCH_NB_LIST(X)
 #undef X
