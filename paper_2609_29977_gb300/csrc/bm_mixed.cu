@@ -82,11 +82,13 @@ __global__ void __launch_bounds__(256) k_mixed_bwd(MixedState m, double *x, int 
 // of the next correction's root term X^T rho in tb. The last CTA applies
 // the stopping test.
 template <int NB>
-__global__ void __launch_bounds__(256, 5) k_mixed_residual(MixedState m, const double *__restrict__ r,
+__global__ void __launch_bounds__(256, FFCfg<NB>::STAGED ? 3 : 5) k_mixed_residual(MixedState m, const double *__restrict__ r,
                                                          const double *__restrict__ x, int iter, int max_iter,
                                                          double tol, cudaGraphConditionalHandle cond) {
+  extern __shared__ __align__(16) float sE[];
   __shared__ unsigned sroot;
   pdl_wait();
+  pdl_trigger();
   if (ir_done(m.ctl)) return;
   const int it = ir_iter(m.ctl, iter);
   const long nrow = (long)m.S * m.N * NB;
@@ -95,12 +97,9 @@ __global__ void __launch_bounds__(256, 5) k_mixed_residual(MixedState m, const d
   const bool ffr = m.ffres && __ldcg(&m.status->ffbad) == 0;
   float om = 0.0f;
   if (ffr) {
-    for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < nrow; e += (long)gridDim.x * blockDim.x) {
-      const long br = e / NB;
-      const int i = (int)(e - br * NB);
-      const int s = (int)(br / m.N), k = (int)(br - (long)s * m.N);
-      om = fmaxf(om, residual_row_ff<NB>(m, r, x, s, k, i));
-    }
+    const int warp = threadIdx.x >> 5;
+    for (long e0 = (long)blockIdx.x * blockDim.x + 32 * warp; e0 < nrow; e0 += (long)gridDim.x * blockDim.x)
+      om = fmaxf(om, residual_rows_ff<NB>(m, r, x, e0, nrow, sE + warp * 2 * FFCfg<NB>::PLANE));
   } else {
     for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < nrow; e += (long)gridDim.x * blockDim.x) {
       const long br = e / NB;
@@ -245,16 +244,20 @@ __global__ void __launch_bounds__(256) k_x_split(MixedState m, const double *__r
 template <int NB>
 __global__ void __launch_bounds__(256) k_residual_out(MixedState m, const double *__restrict__ r,
                                                        const double *__restrict__ x) {
+  extern __shared__ __align__(16) float sE[];
   const long nrow = (long)m.S * m.N * NB;
   const bool ffr = m.ffres && __ldcg(&m.status->ffbad) == 0;
-  for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < nrow; e += (long)gridDim.x * blockDim.x) {
-    const long br = e / NB;
-    const int i = (int)(e - br * NB);
-    const int s = (int)(br / m.N), k = (int)(br - (long)s * m.N);
-    if (ffr)
-      residual_row_ff<NB>(m, r, x, s, k, i);
-    else
+  if (ffr) {
+    const int warp = threadIdx.x >> 5;
+    for (long e0 = (long)blockIdx.x * blockDim.x + 32 * warp; e0 < nrow; e0 += (long)gridDim.x * blockDim.x)
+      residual_rows_ff<NB>(m, r, x, e0, nrow, sE + warp * 2 * FFCfg<NB>::PLANE);
+  } else {
+    for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < nrow; e += (long)gridDim.x * blockDim.x) {
+      const long br = e / NB;
+      const int i = (int)(e - br * NB);
+      const int s = (int)(br / m.N), k = (int)(br - (long)s * m.N);
       residual_row<NB>(m, r, x, s, k, i);
+    }
   }
   for (int c = blockIdx.x; c < m.nr; c += gridDim.x) residual_root_row(m, r, x, NB, c);
 }
@@ -347,7 +350,7 @@ void launch_iteration(const MixedState &m, const double *r, double *x, int iter,
   launch_cluster(k_mixed_fwd<NB>, grid, 256, CS, pdl, st, m, r, x, iter, CS, cond);
   launch_cluster(k_mixed_bwd<NB>, grid, 256, CS, pdl, st, m, x, iter, CS);
   const int blocks = xt_blocks(m.S, m.N, NB, m.nr);
-  launch_plain(k_mixed_residual<NB>, (unsigned)blocks, 256, 0, pdl, st, m, r, (const double *)x, iter, max_iter, tol,
+  launch_plain(k_mixed_residual<NB>, (unsigned)blocks, 256, FFCfg<NB>::bytes, pdl, st, m, r, (const double *)x, iter, max_iter, tol,
                cond);
 }
 
@@ -499,6 +502,13 @@ cudaError_t mixed_prepare(int nb, int nr) {
   if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorUnknown;
   if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
   cudaError_t e = tail_factor_prepare();
+#define X(n)                                                                                                  \
+  if (e == cudaSuccess)                                                                                       \
+    e = cudaFuncSetAttribute(k_mixed_residual<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);    \
+  if (e == cudaSuccess)                                                                                       \
+    e = cudaFuncSetAttribute(k_residual_out<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
+  BM_TAIL_NB_LIST(X)
+#undef X
   if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
   return e;
 }
@@ -699,7 +709,7 @@ void mixed_launch_residual(MixedState *m, const double *r, const double *x, doub
   switch (m->nb) {
 #define X(n)                                                        \
   case n:                                                           \
-    k_residual_out<n><<<(unsigned)blocks, 256, 0, st>>>(c, r, x); \
+    k_residual_out<n><<<(unsigned)blocks, 256, FFCfg<n>::bytes, st>>>(c, r, x); \
     break;
     BM_TAIL_NB_LIST(X)
 #undef X

@@ -4,6 +4,7 @@
 
 #include "bm_ff.cuh"
 #include "bm_tail_factor.cuh"
+#include "bm_tail_rows.cuh"
 
 namespace bm {
 
@@ -577,11 +578,13 @@ constexpr double kFFBeta = 4e-12;
 // stopping test then still accepts omega up to 0.6 tol.
 constexpr double kFFMinTol = 1e-11;
 
+// NB terms: K's entries at kh/kl[t * STRIDE] (global or shared memory), x's
+// contiguous; groups of four per load where both allow it.
 template <int NB, int STRIDE>
 __device__ __forceinline__ void ff_block(double &acc, float &w, const float *__restrict__ kh,
                                          const float *__restrict__ kl, const float *__restrict__ xh,
                                          const float *__restrict__ xl) {
-  constexpr bool V4 = STRIDE == 1 && NB % 4 == 0;
+  constexpr bool V4 = NB % 4 == 0;
 #pragma unroll
   for (int j0 = 0; j0 < NB; j0 += 8) {
     constexpr int CH = 8;
@@ -591,12 +594,20 @@ __device__ __forceinline__ void ff_block(double &acc, float &w, const float *__r
 #pragma unroll
       for (int g = 0; g < CH / 4; ++g) {
         if (4 * g < cnt) {
-          const float4 va = *reinterpret_cast<const float4 *>(kh + j0 + 4 * g);
-          const float4 vl = *reinterpret_cast<const float4 *>(kl + j0 + 4 * g);
+          if constexpr (STRIDE == 1) {
+            const float4 va = *reinterpret_cast<const float4 *>(kh + j0 + 4 * g);
+            const float4 vl = *reinterpret_cast<const float4 *>(kl + j0 + 4 * g);
+            a[4 * g] = va.x; a[4 * g + 1] = va.y; a[4 * g + 2] = va.z; a[4 * g + 3] = va.w;
+            al[4 * g] = vl.x; al[4 * g + 1] = vl.y; al[4 * g + 2] = vl.z; al[4 * g + 3] = vl.w;
+          } else {
+#pragma unroll
+            for (int t = 4 * g; t < 4 * g + 4; ++t) {
+              a[t] = kh[(j0 + t) * STRIDE];
+              al[t] = kl[(j0 + t) * STRIDE];
+            }
+          }
           const float4 vb = __ldg(reinterpret_cast<const float4 *>(xh + j0 + 4 * g));
           const float4 vc = __ldg(reinterpret_cast<const float4 *>(xl + j0 + 4 * g));
-          a[4 * g] = va.x; a[4 * g + 1] = va.y; a[4 * g + 2] = va.z; a[4 * g + 3] = va.w;
-          al[4 * g] = vl.x; al[4 * g + 1] = vl.y; al[4 * g + 2] = vl.z; al[4 * g + 3] = vl.w;
           b[4 * g] = vb.x; b[4 * g + 1] = vb.y; b[4 * g + 2] = vb.z; b[4 * g + 3] = vb.w;
           bl[4 * g] = vc.x; bl[4 * g + 1] = vc.y; bl[4 * g + 2] = vc.z; bl[4 * g + 3] = vc.w;
         }
@@ -630,27 +641,84 @@ __device__ __forceinline__ void ff_block(double &acc, float &w, const float *__r
   }
 }
 
-// Row i of block row (s, k) of the residual in float-float; as
-// residual_row, but (|K||x|)_i from the hi parts (scaled down by 2^-22 to
-// cover their rounding, so omega is never understated).
+// Shared memory of the float-float residual for wide blocks: per warp 32 rows
+// of E (hi and lo planes) of CW columns at a time, row stride an odd number of
+// 16-byte groups. Smaller blocks read the rows directly (below).
 template <int NB>
-__device__ __forceinline__ float residual_row_ff(const MixedState &m, const double *__restrict__ r,
-                                                 const double *__restrict__ x, int s, int k, int i) {
-  constexpr int NB2 = NB * NB;
+struct FFCfg {
+  static constexpr bool STAGED = NB > 32;
+  static constexpr int CW = NB > 32 ? NB / 2 : NB;
+  static constexpr int LD = CW / 4 % 2 ? CW : CW + 4;
+  static constexpr int PLANE = 32 * LD;
+  static constexpr size_t bytes = STAGED ? (size_t)8 * 2 * PLANE * sizeof(float) : 0;   // eight warps
+};
+
+// 32 consecutive rows e0 + lane of the residual over all tails in
+// float-float (row e = block row (s, k), row i in it); as residual_row, but
+// (|K||x|)_i from the hi parts (scaled down by 2^-22 to cover their rounding,
+// so omega is never understated). Returns the lane's omega (0 beyond nrow).
+// buf: 2 * FFCfg<NB>::PLANE floats of the warp.
+//
+// For wide blocks D's row i is read as column i of the symmetric block,
+// contiguous over the lanes (the same values in the same order), and the
+// rows of E_k that 32 consecutive rows need, contiguous in memory, arrive
+// through shared memory by asynchronous copies behind D's part: nb = 48,
+// S = 512, N = 256: 1536 -> 1295 us per pass. With nb = 24 (S = 512, N = 128) the
+// same takes 180 instead of 170 us, and D by columns alone 189: a row is 96
+// bytes there, six 16-byte loads hit the lines that the first one fetched,
+// and 48 scalar loads cost more than they save.
+template <int NB>
+__device__ __forceinline__ float residual_rows_ff(const MixedState &m, const double *__restrict__ r,
+                                                  const double *__restrict__ x, long e0, long nrow, float *buf) {
+  constexpr int NB2 = NB * NB, CW = FFCfg<NB>::CW, LD = FFCfg<NB>::LD, Q = CW / 4;
+  const int lane = threadIdx.x & 31;
+  const long e = e0 + lane;
+  const bool ok = e < nrow;
   const int N = m.N, nr = m.nr;
   const size_t n0 = (size_t)m.S * N * NB;
-  const long br = (long)s * N + k;
+  const long br = e / NB;
+  const int i = (int)(e - br * NB), s = (int)(br / N), k = (int)(br - (long)s * N);
   const size_t off = (size_t)br * NB;
+  // row of E (NB floats each) that is this row's left block, -1 if none
+  const long erow = ok && k > 0 ? e - (long)(s + 1) * NB : -1;
+  float *bh = buf, *bl = buf + FFCfg<NB>::PLANE;
+  auto stage_e = [&](int c0) {
+#pragma unroll
+    for (int u = 0; u < Q; ++u) {
+      const int t = lane + 32 * u, row = t / Q, c = 4 * (t - row * Q);
+      const long src = __shfl_sync(0xffffffffu, erow, row);
+      if (src >= 0) {
+        rows::cp_async16(bh + row * LD + c, m.Keh + src * NB + c0 + c);
+        rows::cp_async16(bl + row * LD + c, m.Kel + src * NB + c0 + c);
+      }
+    }
+  };
+  if constexpr (FFCfg<NB>::STAGED) stage_e(0);
   double acc = 0.0;
   float w = 0.0f;
-  {
-    const size_t kb = (size_t)br * NB2 + (size_t)i * NB;
-    ff_block<NB, 1>(acc, w, m.Kdh + kb, m.Kdl + kb, m.xh + off, m.xl + off);
+  if (ok) {
+    if constexpr (FFCfg<NB>::STAGED) {
+      const size_t kb = (size_t)br * NB2 + i;   // column i of the symmetric block
+      ff_block<NB, NB>(acc, w, m.Kdh + kb, m.Kdl + kb, m.xh + off, m.xl + off);
+    } else {
+      const size_t kb = (size_t)br * NB2 + (size_t)i * NB;
+      ff_block<NB, 1>(acc, w, m.Kdh + kb, m.Kdl + kb, m.xh + off, m.xl + off);
+    }
   }
-  if (k > 0) {   // block (k, k-1) = E_k: row i
-    const size_t eb = ((size_t)s * (N - 1) + (k - 1)) * NB2 + (size_t)i * NB;
-    ff_block<NB, 1>(acc, w, m.Keh + eb, m.Kel + eb, m.xh + off - NB, m.xl + off - NB);
+  if constexpr (FFCfg<NB>::STAGED) {   // block (k, k-1) = E_k: row i
+#pragma unroll
+    for (int c0 = 0; c0 < NB; c0 += CW) {
+      rows::cp_async_wait();
+      __syncwarp();
+      if (erow >= 0)
+        ff_block<CW, 1>(acc, w, bh + lane * LD, bl + lane * LD, m.xh + off - NB + c0, m.xl + off - NB + c0);
+      __syncwarp();
+      if (c0 + CW < NB) stage_e(c0 + CW);
+    }
+  } else if (erow >= 0) {
+    ff_block<NB, 1>(acc, w, m.Keh + erow * NB, m.Kel + erow * NB, m.xh + off - NB, m.xl + off - NB);
   }
+  if (!ok) return 0.0f;
   if (k + 1 < N) {   // block (k, k+1) = E_{k+1}^T: column i of E_{k+1}
     const size_t eb = ((size_t)s * (N - 1) + k) * NB2 + i;
     ff_block<NB, NB>(acc, w, m.Keh + eb, m.Kel + eb, m.xh + off + NB, m.xl + off + NB);
