@@ -51,11 +51,30 @@ void mixed_launch_export(MixedState *m, double *Ld, double *Ll, double *Lr, doub
 
 using namespace bm;
 
-// Chunks of tails whose host-to-device copies the pipelined host entry
-// overlaps with the factor (measured on GB300, mixed workload, copies
-// 2.93 ms: 2 chunks 8.76 ms per call, 4: 8.22, 8: 7.93, 16: 9.26; serial
-// 10.0 ms).
+// Pipelined host entry: the tails' blocks are copied in chunks, and the first
+// grid-wide levels run per chunk behind its copy. More chunks hide more of
+// the factor behind the copies, but a launch that does not fill the GPU costs
+// nearly as much as one that does, so there is a chunk for every 2500
+// positions of level 0 (at least 2, at most 8), and the levels that run per
+// chunk are those with 1500 tasks in it (level 0 always). Measured, us per
+// call by (chunks, levels per chunk):
+//   S=512 N=128 nb=24:  (8,1) 5885 (8,2) 5118 (8,3) 4859 (8,4) 5060 (4,3) 5007 (16,3) 5488, copies first 6762
+//   S=100 N=160 nb=16:  (8,1) 939 (3,1) 938 (3,2) 888 (3,3) 902 (4,2) 896, copies first 1007
+//   S=64  N=64  nb=12:  (8,1) 383 (4,1) 313 (2,1) 297, copies first 300
+//   S=60  N=40  nb=48:  (8,1) 2539 (4,1) 2105 (2,1) 2048 (2,2) 2085, copies first 2229
 static constexpr int kHostChunks = 8;
+static constexpr long kChunkTasks = 2500, kChunkLevelTasks = 1500;
+
+static int host_chunks(int S, int N) {
+  const long k = (long)S * (N / 2) / kChunkTasks;
+  const int K = k < 2 ? 2 : k > kHostChunks ? kHostChunks : (int)k;
+  return K < S ? K : S;
+}
+static int host_chunk_levels(int S, int N, int K, int top) {
+  int l = top < 1 ? top : 1;
+  while (l < top && (long)S / K * (((N - 1) >> l) + 1) >= kChunkLevelTasks) ++l;
+  return l;
+}
 
 struct GraphSlot {
   cudaGraphExec_t exec = nullptr;
@@ -506,12 +525,9 @@ static bool host_pinned(const void *p) {
 
 // The factor of the host entry with its copies pipelined (FP64 tails with
 // compile-time kernels, a schedule already chosen, page-locked inputs): the
-// tails' blocks are copied in kHostChunks chunks on a second stream, and the
-// first grid-wide level of a chunk runs as soon as its blocks have arrived,
-// so the transfer of later chunks overlaps the factor of earlier ones (one
-// chunk's level 0 takes about as long as its copy; running level 1 per
-// chunk as well measured slower: 8.97 against 7.93 ms per call on the mixed
-// workload, the smaller level-1 grids filling the SMs less well). The
+// tails' blocks are copied in chunks on a second stream, and the first
+// grid-wide levels of a chunk run as soon as its blocks have arrived, so the
+// transfer of later chunks overlaps the factor of earlier ones. The
 // remaining levels run over all tails once the last chunk has arrived, and
 // the top kernel (whose last CTA does the root step) once C, R and r have. Every block
 // is computed by the same kernels in the same order as in bm_factor, so the
@@ -538,8 +554,7 @@ static bool factor_host_pipelined(bm_handle h, const double *hD, const double *h
   }
   const int S = d.S, N = d.N, nb = d.nb, nr = d.nr;
   const size_t b2 = (size_t)nb * nb, n = (size_t)S * N * nb + nr;
-  const int K = S < kHostChunks ? S : kHostChunks;
-  const int lp = h->sched.top < 1 ? h->sched.top : 1;
+  const int K = host_chunks(S, N), lp = host_chunk_levels(S, N, K, h->sched.top);
   F64View v = h->v;
   v.D = h->sD; v.E = N > 1 ? h->sE : nullptr; v.C = h->sC; v.R = h->sR;
   const TailSched *sc = &h->sched;
