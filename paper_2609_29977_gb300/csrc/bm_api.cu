@@ -22,7 +22,7 @@ void f64_launch_factor(const F64View &v, cudaStream_t st, const TailSched *sc = 
 bool f64_tune(const F64View &v, cudaStream_t st, TailSched *out);
 bool tune_cache_lookup(const std::string &key, std::vector<int> &vals);
 void tune_cache_store(const std::string &key, const std::vector<int> &vals);
-void f64_launch_solve(const F64View &v, const double *r, double *x, cudaStream_t st);
+void f64_launch_solve(const F64View &v, const double *r, double *x, double *r0t, cudaStream_t st);
 void f64_launch_export_ld(const F64View &v, double *Ld, cudaStream_t st);
 void f64_launch_factor_part(const F64View &v, int s0, int s1, int lo, int hi, bool top, cudaStream_t st,
                             const TailSched *sc);
@@ -41,13 +41,10 @@ void mixed_launch_factor(MixedState *m, const double *D, const double *E, const 
                          cudaStream_t st);
 // body_st non-null: st is capturing, and the refinement loop becomes a
 // conditional graph node whose body is captured from body_st (programmatic
-// launches inside the body when body_pdl is set). Launched directly, only the
-// first `unroll` iterations are, and the resumption of a failed refinement
-// only with resume: a solve cut short that way leaves status->more set, or
-// its code BM_ERR_NOT_CONVERGED.
+// launches inside the body when body_pdl is set).
 cudaError_t mixed_launch_solve(MixedState *m, const double *r, double *x, int max_refine, double tol,
                                cudaStream_t st, cudaStream_t body_st, cudaStream_t if_st, cudaStream_t body2_st,
-                               bool body_pdl, int unroll = 1 << 30, bool resume = true);
+                               bool body_pdl);
 void mixed_launch_export(MixedState *m, double *Ld, double *Ll, double *Lr, double *F, double *LR,
                          cudaStream_t st);
 }  // namespace bm
@@ -92,6 +89,7 @@ struct bm_handle_s {
   size_t pool_bytes = 0;
   bool owns_pool = true;
   F64View v{};           // FP64 buffers (unused pointers null in mixed mode)
+  double *r0t = nullptr; // [nr] root right-hand side scratch
   Status *status = nullptr;
   unsigned *tickets = nullptr;
   MixedState *mixed = nullptr;
@@ -151,6 +149,7 @@ static size_t f64_bytes(int S, int N, int nb, int nr) {
   t += align_up((size_t)nr * nr * sizeof(double), 256) * 2;  // LR Rt
   t += align_up(SN * nb * sizeof(double), 256) * 3;          // invd y zt
   t += align_up((size_t)S * nr * sizeof(double), 256);       // tb
+  t += align_up((size_t)nr * sizeof(double), 256);           // r0t
   return t;
 }
 
@@ -233,6 +232,7 @@ bm_status analyze_impl(const bm_desc *desc, void *mem, size_t bytes, cudaStream_
     v.LR = take((size_t)nr * nr * 8); v.Rt = take((size_t)nr * nr * 8);
     v.invd = take(SN * nb * 8); v.y = take(SN * nb * 8); v.zt = take(SN * nb * 8);
     v.tb = take((size_t)S * nr * 8);
+    h->r0t = take((size_t)nr * 8);
     v.tickets = h->tickets;
     v.status = h->status;
     if (f64_prepare(nb, nr) != cudaSuccess) goto cuda_fail;
@@ -440,17 +440,9 @@ extern "C" bm_status bm_solve(bm_handle h, const double *r, double *x, void *str
     return s;
   }
   F64View v = h->v;
+  double *r0t = h->r0t;
   const void *key[2] = {r, x};
-  return run(h, h->gsol, key, 2, st, [&](cudaStream_t cs, bool) { f64_launch_solve(v, r, x, cs); });
-}
-
-// bm_solve of a directly launched mixed handle with its first `unroll`
-// iterations only and without the resumption of a failed refinement.
-bm_status solve_short(bm_handle h, const double *r, double *x, cudaStream_t st, int unroll) {
-  const cudaError_t e = mixed_launch_solve(h->mixed, r, x, h->desc.max_refine, h->desc.tol, st, nullptr, nullptr,
-                                           nullptr, false, unroll, false);
-  cudaGetLastError();
-  return e == cudaSuccess ? BM_OK : BM_ERR_CUDA;
+  return run(h, h->gsol, key, 2, st, [&](cudaStream_t cs, bool) { f64_launch_solve(v, r, x, r0t, cs); });
 }
 
 extern "C" bm_status bm_residual(bm_handle h, const double *r, const double *x, double *rho, void *stream) {
