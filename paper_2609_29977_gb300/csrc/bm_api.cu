@@ -22,7 +22,7 @@ void f64_launch_factor(const F64View &v, cudaStream_t st, const TailSched *sc = 
 bool f64_tune(const F64View &v, cudaStream_t st, TailSched *out);
 bool tune_cache_lookup(const std::string &key, std::vector<int> &vals);
 void tune_cache_store(const std::string &key, const std::vector<int> &vals);
-void f64_launch_solve(const F64View &v, const double *r, double *x, double *r0t, cudaStream_t st);
+void f64_launch_solve(const F64View &v, const double *r, double *x, cudaStream_t st);
 void f64_launch_export_ld(const F64View &v, double *Ld, cudaStream_t st);
 void f64_launch_factor_part(const F64View &v, int s0, int s1, int lo, int hi, bool top, cudaStream_t st,
                             const TailSched *sc);
@@ -89,7 +89,6 @@ struct bm_handle_s {
   size_t pool_bytes = 0;
   bool owns_pool = true;
   F64View v{};           // FP64 buffers (unused pointers null in mixed mode)
-  double *r0t = nullptr; // [nr] root right-hand side scratch
   Status *status = nullptr;
   unsigned *tickets = nullptr;
   MixedState *mixed = nullptr;
@@ -149,7 +148,6 @@ static size_t f64_bytes(int S, int N, int nb, int nr) {
   t += align_up((size_t)nr * nr * sizeof(double), 256) * 2;  // LR Rt
   t += align_up(SN * nb * sizeof(double), 256) * 3;          // invd y zt
   t += align_up((size_t)S * nr * sizeof(double), 256);       // tb
-  t += align_up((size_t)nr * sizeof(double), 256);           // r0t
   return t;
 }
 
@@ -232,7 +230,6 @@ bm_status analyze_impl(const bm_desc *desc, void *mem, size_t bytes, cudaStream_
     v.LR = take((size_t)nr * nr * 8); v.Rt = take((size_t)nr * nr * 8);
     v.invd = take(SN * nb * 8); v.y = take(SN * nb * 8); v.zt = take(SN * nb * 8);
     v.tb = take((size_t)S * nr * 8);
-    h->r0t = take((size_t)nr * 8);
     v.tickets = h->tickets;
     v.status = h->status;
     if (f64_prepare(nb, nr) != cudaSuccess) goto cuda_fail;
@@ -440,9 +437,8 @@ extern "C" bm_status bm_solve(bm_handle h, const double *r, double *x, void *str
     return s;
   }
   F64View v = h->v;
-  double *r0t = h->r0t;
   const void *key[2] = {r, x};
-  return run(h, h->gsol, key, 2, st, [&](cudaStream_t cs, bool) { f64_launch_solve(v, r, x, r0t, cs); });
+  return run(h, h->gsol, key, 2, st, [&](cudaStream_t cs, bool) { f64_launch_solve(v, r, x, cs); });
 }
 
 extern "C" bm_status bm_residual(bm_handle h, const double *r, const double *x, double *rho, void *stream) {

@@ -29,6 +29,7 @@
 #include <mutex>
 
 #include "bm_root.cuh"
+#include "bm_team.cuh"
 
 namespace bm {
 namespace {
@@ -75,19 +76,6 @@ __device__ void cta_trsm_lt(double *X, int m, const double *L, const double *inv
     }
     __syncthreads();
   }
-}
-
-// Fixed-order CTA sum of one value per thread (blockDim.x a power of two).
-__device__ double cta_sum(double v, double *red) {
-  red[threadIdx.x] = v;
-  for (int w = blockDim.x >> 1; w > 0; w >>= 1) {
-    __syncthreads();
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-  }
-  __syncthreads();
-  const double t = red[0];
-  __syncthreads();
-  return t;
 }
 
 // ---------------------------------------------------------------------------
@@ -351,36 +339,51 @@ __global__ void k_solve_x1_fwd(F64View v, const double *__restrict__ r) {
   }
 }
 
-// Root: r~_0 = r_0 - sum_i t_i (one CTA per component, fixed order); the
-// last CTA solves L_R L_R^T x_0 = r~_0 and writes x_0.
-__global__ void k_solve_root(F64View v, const double *__restrict__ r, double *__restrict__ x,
-                             double *__restrict__ r0t) {
-  __shared__ double red[256];
-  __shared__ double sR[64 * 64 + 64 + 64];
-  __shared__ int last;
-  const int nr = v.nr, S = v.S, i = blockIdx.x;
+// Root: r~_0 = r_0 - sum_i t_i (one warp per component, in the order of
+// root_sum_warp), then L_R L_R^T x_0 = r~_0 by one warp, a row per lane (and
+// row + 32 for nr > 32), and x_0. One CTA: with one per component and an
+// election of the last, block-wide sums and substitutions took 7 to 12 us
+// (nr = 2 to 16) of a chain whose arithmetic takes one to three
+// (S = 4, N = 16, nb = 4: factor and solve 56.2 -> 53.9 us).
+__global__ void __launch_bounds__(512) k_solve_root(F64View v, const double *__restrict__ r,
+                                                    double *__restrict__ x) {
+  __shared__ double sL[64 * 65], sz[64], sInv[64];
+  const int nr = v.nr, S = v.S, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const size_t n0 = (size_t)S * v.N * v.nb;
-  double acc = 0.0;
-  for (int s = threadIdx.x; s < S; s += blockDim.x) acc += v.tb[(size_t)s * nr + i];
-  const double tot = cta_sum(acc, red);
-  if (threadIdx.x == 0) {
-    r0t[i] = r[n0 + i] - tot;
-    __threadfence();
-    last = (atomicAdd(&v.tickets[1], 1u) == gridDim.x - 1);
+  pdl_wait();
+  for (int e = threadIdx.x; e < nr * nr; e += blockDim.x) {
+    const int i = e / nr, j = e - i * nr;
+    sL[i * 65 + j] = v.LR[e];
+    if (i == j) sInv[i] = 1.0 / v.LR[e];
+  }
+  for (int c = warp; c < nr; c += blockDim.x >> 5) {
+    double acc = 0.0;
+#pragma unroll 4
+    for (int s = lane; s < S; s += 32) acc += __ldcg(v.tb + (size_t)s * nr + c);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) sz[c] = r[n0 + c] - acc;
   }
   __syncthreads();
-  if (!last) return;
-  __threadfence();
-  double *sL = sR, *sz = sR + nr * nr, *sInv = sz + nr;
-  for (int e = threadIdx.x; e < nr * nr; e += blockDim.x) sL[e] = __ldcg(v.LR + e);
-  for (int e = threadIdx.x; e < nr; e += blockDim.x) sz[e] = __ldcg(r0t + e);
-  __syncthreads();
-  for (int e = threadIdx.x; e < nr; e += blockDim.x) sInv[e] = 1.0 / sL[e * nr + e];
-  __syncthreads();
-  cta_trsv_l(sz, sL, sInv, nr);
-  cta_trsv_lt(sz, sL, sInv, nr);
-  for (int e = threadIdx.x; e < nr; e += blockDim.x) x[n0 + e] = sz[e];
-  if (threadIdx.x == 0) v.tickets[1] = 0u;
+  if (warp != 0) return;
+  const int i1 = lane + 32;
+  double z0 = lane < nr ? sz[lane] : 0.0, z1 = i1 < nr ? sz[i1] : 0.0;
+  for (int j = 0; j < nr; ++j) {
+    const double zj = __shfl_sync(0xffffffffu, j < 32 ? z0 : z1, j & 31) * sInv[j];
+    if (lane == j) z0 = zj;
+    if (i1 == j) z1 = zj;
+    if (lane > j && lane < nr) z0 = fma(-sL[lane * 65 + j], zj, z0);
+    if (i1 > j && i1 < nr) z1 = fma(-sL[i1 * 65 + j], zj, z1);
+  }
+  for (int j = nr - 1; j >= 0; --j) {
+    const double zj = __shfl_sync(0xffffffffu, j < 32 ? z0 : z1, j & 31) * sInv[j];
+    if (lane == j) z0 = zj;
+    if (i1 == j) z1 = zj;
+    if (lane < j) z0 = fma(-sL[j * 65 + lane], zj, z0);
+    if (i1 < j) z1 = fma(-sL[j * 65 + i1], zj, z1);
+  }
+  if (lane < nr) x[n0 + lane] = z0;
+  if (i1 < nr) x[n0 + i1] = z1;
 }
 
 // Root propagation y_1 -= F_{i,1}^T x_0 and x_1 = L_{i,1}^{-T} y_1.
@@ -444,7 +447,7 @@ size_t f64_factor_smem(int nb, int nr) {
 }
 
 bool f64_cluster_solve_supported(int nb);
-void f64_cluster_launch_solve(const F64View &v, const double *r, double *x, double *r0t, cudaStream_t st);
+void f64_cluster_launch_solve(const F64View &v, const double *r, double *x, cudaStream_t st);
 
 // The dynamic shared-memory limit is a per-kernel attribute shared by every
 // handle in the process, so it is always raised to what the largest
@@ -570,13 +573,13 @@ void f64_launch_export_ld(const F64View &v, double *Ld, cudaStream_t st) {
   k_copy_lower<<<(unsigned)blocks, 256, 0, st>>>(v.Ld, Ld, n, v.nb);
 }
 
-void f64_launch_solve_root(const F64View &v, const double *r, double *x, double *r0t, cudaStream_t st) {
-  k_solve_root<<<v.nr, 256, 0, st>>>(v, r, x, r0t);
+void f64_launch_solve_root(const F64View &v, const double *r, double *x, cudaStream_t st) {
+  launch_pdl(k_solve_root, 1u, 32u * (v.nr < 16 ? v.nr : 16), 0, st, v, r, x);
 }
 
-void f64_launch_solve(const F64View &v, const double *r, double *x, double *r0t, cudaStream_t st) {
+void f64_launch_solve(const F64View &v, const double *r, double *x, cudaStream_t st) {
   if (f64_cluster_solve_supported(v.nb)) {
-    f64_cluster_launch_solve(v, r, x, r0t, st);
+    f64_cluster_launch_solve(v, r, x, st);
     return;
   }
   const int T = solve_threads(v.nb);
@@ -586,7 +589,7 @@ void f64_launch_solve(const F64View &v, const double *r, double *x, double *r0t,
     k_solve_fwd_level<<<grid, T, smem, st>>>(v, r, l);
   }
   k_solve_x1_fwd<<<v.S, T, smem, st>>>(v, r);
-  k_solve_root<<<v.nr, 256, 0, st>>>(v, r, x, r0t);
+  f64_launch_solve_root(v, r, x, st);
   k_solve_x1_bwd<<<v.S, T, smem, st>>>(v, x);
   for (int l = v.Lc - 1; l >= 0; --l) {
     dim3 grid(level_elims(v.N, l), v.S);

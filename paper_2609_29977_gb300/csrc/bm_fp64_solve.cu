@@ -268,7 +268,7 @@ cudaError_t launch_bwd_kernel(const F64View &v, double *x, cudaStream_t st) {
 
 }  // namespace
 
-void f64_launch_solve_root(const F64View &v, const double *r, double *x, double *r0t, cudaStream_t st);
+void f64_launch_solve_root(const F64View &v, const double *r, double *x, cudaStream_t st);
 
 // The cluster solves substitute with the scaled unit factor that the
 // compile-time tail factor stores above each diagonal block's diagonal, so
@@ -285,13 +285,13 @@ bool f64_cluster_solve_supported(int nb) {
   return false;
 }
 
-void f64_cluster_launch_solve(const F64View &v, const double *r, double *x, double *r0t, cudaStream_t st) {
+void f64_cluster_launch_solve(const F64View &v, const double *r, double *x, cudaStream_t st) {
   switch (v.nb) {
 #define X(n)                                                    \
   case n:                                                       \
     launch_tail_kernel<n>(solve_capped(v.S, pick_cluster(v.S)) ? k_solve_fwd_tail<n, SolveCfg<n>::MINB> \
                                                                : k_solve_fwd_tail<n, 1>, v, r, st); \
-    f64_launch_solve_root(v, r, x, r0t, st);                    \
+    f64_launch_solve_root(v, r, x, st);                         \
     launch_bwd_kernel<n>(v, x, st);                             \
     break;
     BM_SOLVE_NB_LIST(X)

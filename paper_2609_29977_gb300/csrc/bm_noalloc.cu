@@ -32,7 +32,7 @@ namespace bm {
 size_t f64_factor_smem(int nb, int nr);
 cudaError_t f64_prepare(int nb, int nr);
 void f64_launch_factor(const F64View &v, cudaStream_t st, const TailSched *sc = nullptr);
-void f64_launch_solve(const F64View &v, const double *r, double *x, double *r0t, cudaStream_t st);
+void f64_launch_solve(const F64View &v, const double *r, double *x, cudaStream_t st);
 }  // namespace bm
 
 using namespace bm;
@@ -55,7 +55,6 @@ size_t noalloc_bytes(int S, int N, int nb, int nr) {
   t += align_up((size_t)nr * nr * sizeof(double), 256) * 2;  // LR Rt
   t += align_up(SN * nb * sizeof(double), 256) * 3;          // invd y zt
   t += align_up((size_t)S * nr * sizeof(double), 256);       // tb
-  t += align_up((size_t)nr * sizeof(double), 256);           // r0t
   return t;
 }
 
@@ -118,7 +117,6 @@ extern "C" bm_status bm_factor_solve_noalloc(int S, int N, int nb, int nr, const
   v.LR = take((size_t)nr * nr * 8); v.Rt = take((size_t)nr * nr * 8);
   v.invd = take(SN * nb * 8); v.y = take(SN * nb * 8); v.zt = take(SN * nb * 8);
   v.tb = take((size_t)S * nr * 8);
-  double *r0t = take((size_t)nr * 8);
   v.status = (Status *)base;
   v.tickets = (unsigned *)((char *)base + 256);
 
@@ -128,7 +126,7 @@ extern "C" bm_status bm_factor_solve_noalloc(int S, int N, int nb, int nr, const
     return BM_ERR_CUDA;
   }
   f64_launch_factor(v, st);
-  f64_launch_solve(v, r, x, r0t, st);
+  f64_launch_solve(v, r, x, st);
   if (cudaGetLastError() != cudaSuccess) return BM_ERR_CUDA;
   Status hs;
   if (cudaMemcpyAsync(&hs, base, sizeof(Status), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
