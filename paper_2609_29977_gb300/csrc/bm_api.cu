@@ -41,10 +41,13 @@ void mixed_launch_factor(MixedState *m, const double *D, const double *E, const 
                          cudaStream_t st);
 // body_st non-null: st is capturing, and the refinement loop becomes a
 // conditional graph node whose body is captured from body_st (programmatic
-// launches inside the body when body_pdl is set).
+// launches inside the body when body_pdl is set). Launched directly, only the
+// first `unroll` iterations are, and the resumption of a failed refinement
+// only with resume: a solve cut short that way leaves status->more set, or
+// its code BM_ERR_NOT_CONVERGED.
 cudaError_t mixed_launch_solve(MixedState *m, const double *r, double *x, int max_refine, double tol,
                                cudaStream_t st, cudaStream_t body_st, cudaStream_t if_st, cudaStream_t body2_st,
-                               bool body_pdl);
+                               bool body_pdl, int unroll = 1 << 30, bool resume = true);
 void mixed_launch_export(MixedState *m, double *Ld, double *Ll, double *Lr, double *F, double *LR,
                          cudaStream_t st);
 }  // namespace bm
@@ -439,6 +442,15 @@ extern "C" bm_status bm_solve(bm_handle h, const double *r, double *x, void *str
   F64View v = h->v;
   const void *key[2] = {r, x};
   return run(h, h->gsol, key, 2, st, [&](cudaStream_t cs, bool) { f64_launch_solve(v, r, x, cs); });
+}
+
+// bm_solve of a directly launched mixed handle with its first `unroll`
+// iterations only and without the resumption of a failed refinement.
+bm_status solve_short(bm_handle h, const double *r, double *x, cudaStream_t st, int unroll) {
+  const cudaError_t e = mixed_launch_solve(h->mixed, r, x, h->desc.max_refine, h->desc.tol, st, nullptr, nullptr,
+                                           nullptr, false, unroll, false);
+  cudaGetLastError();
+  return e == cudaSuccess ? BM_OK : BM_ERR_CUDA;
 }
 
 extern "C" bm_status bm_residual(bm_handle h, const double *r, const double *x, double *rho, void *stream) {

@@ -88,7 +88,6 @@ __global__ void __launch_bounds__(256, FFCfg<NB>::STAGED ? 3 : 5) k_mixed_residu
   extern __shared__ __align__(16) float sE[];
   __shared__ unsigned sroot;
   pdl_wait();
-  pdl_trigger();
   if (ir_done(m.ctl)) return;
   const int it = ir_iter(m.ctl, iter);
   const long nrow = (long)m.S * m.N * NB;
@@ -640,7 +639,7 @@ void retry_root(const MixedState &m, cudaStream_t st) {
 
 cudaError_t mixed_launch_solve(MixedState *m, const double *r, double *x, int max_refine, double tol,
                                cudaStream_t st, cudaStream_t body_st, cudaStream_t if_st, cudaStream_t body2_st,
-                               bool body_pdl) {
+                               bool body_pdl, int unroll, bool resume) {
   // reset the per-solve control words
   cudaError_t e = cudaMemsetAsync(m->ctl, 0, sizeof(IRCtl), st);
   if (e != cudaSuccess) return e;
@@ -656,7 +655,7 @@ cudaError_t mixed_launch_solve(MixedState *m, const double *r, double *x, int ma
   }
   // automatic mode: a refinement that fails without refined coupling
   // columns is resumed with them (k_retry_arm)
-  const bool retry = m->cmode == 1;
+  const bool retry = m->cmode == 1 && resume;
   if (body_st) {
     switch (m->nb) {
 #define X(n)                                                                                  \
@@ -669,12 +668,13 @@ cudaError_t mixed_launch_solve(MixedState *m, const double *r, double *x, int ma
     }
     return cudaErrorInvalidValue;
   }
-  for (int it = 0; it <= max_refine; ++it) {
+  for (int it = 0; it <= max_refine && it < unroll; ++it) {
     switch (m->nb) {
 #define X(n)                                                     \
   case n:                                                        \
     launch_iteration<n>(*m, r, x, it, max_refine, tol, st, 0, true); \
     break;
+// unroll, resume: directly launched only, see the declaration in bm_api.cu.
       BM_TAIL_NB_LIST(X)
 #undef X
     }

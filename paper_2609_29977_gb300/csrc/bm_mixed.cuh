@@ -670,7 +670,7 @@ struct FFCfg {
 template <int NB>
 __device__ __forceinline__ float residual_rows_ff(const MixedState &m, const double *__restrict__ r,
                                                   const double *__restrict__ x, long e0, long nrow, float *buf) {
-  constexpr int NB2 = NB * NB, CW = FFCfg<NB>::CW, LD = FFCfg<NB>::LD, Q = CW / 4;
+  constexpr int NB2 = NB * NB, CW = FFCfg<NB>::CW, LD = FFCfg<NB>::LD, Q = CW < 4 ? 1 : CW / 4;
   const int lane = threadIdx.x & 31;
   const long e = e0 + lane;
   const bool ok = e < nrow;
@@ -838,7 +838,9 @@ __device__ __forceinline__ bool ir_stop(const MixedState &m, float root_omega, i
   ctl->omega_prev = omega;
   ctl->wmax = 0u;
   ctl->loop = iter + 1;
-  return ctl->converged == 0;
+  const bool more = ctl->converged == 0;
+  m.status->more = more ? 1 : 0;
+  return more;
 }
 
 // Root rows and the stopping test of one system, by its last CTA.

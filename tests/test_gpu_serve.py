@@ -256,3 +256,40 @@ def test_mixed_failure_falls_back_to_fp64():
     assert st["fallbacks"] == 1 and st["completed"] == 2
     assert np.array_equal(xs[0].cpu().numpy(), fp64_x[0])
     assert comps[0]["t_start_us"] <= comps[0]["t_factor_us"] <= comps[0]["t_done_us"]
+
+
+# barrier 10^+-6 systems whose refinement stalls with the FP32-based root and
+# is resumed with refined coupling columns, and one that takes more
+# corrections than a request's solves launch at first
+@pytest.mark.parametrize("S,N,nb,nr,seed,root,tol", [(2, 12, 24, 8, 46, "wishart", 1e-10),
+                                                     (6, 40, 24, 8, 240, "scaled_identity", 1e-10),
+                                                     (3, 33, 12, 4, 7, "scaled_identity", 1e-16)])
+@pytest.mark.parametrize("host_io", [False, True])
+def test_solves_cut_short_run_again_complete(S, N, nb, nr, seed, root, tol, host_io):
+    """A request's solves launch their first iterations only; what those do
+    not finish runs again, complete, and gives the bits, iteration counts and
+    errors of complete solves of a handle of its own."""
+    import paper_2609_29977_gb300 as bm
+    w = bmgen.Workload("c", S, N, nb, nr, workload_id=94, barrier=(-6.0, 6.0), root=root, shared_A=True)
+    d = bmgen.generate(w, seed=seed)
+    g = torch.Generator().manual_seed(seed)
+    rs = torch.cat([d["r"][None], torch.randn((2, d["r"].numel()), generator=g, dtype=torch.float64)])
+    dev = {k: d[k].cuda() for k in ("D", "E", "C", "R")}
+    solver = bm.BranchKKTSolver(S, N, nb, nr, precision=bm.BM_PREC_FP32_IR, tol=tol, flags=bm.BM_FLAG_NO_GRAPH)
+    solver.factor(dev["D"], dev["E"], dev["C"], dev["R"])
+    ref, infos = [], []
+    for r in rs:
+        ref.append(solver.solve(r.cuda()).cpu())
+        infos.append(solver.query())
+    solver.close()
+    assert infos[0]["coupling_refined"] == 1 or infos[0]["iters"] >= 5 or infos[0]["status"] == 5
+    server = bm.BranchKKTServer(1 << 28, slots=2, tol=tol)
+    src = {k: d[k].pin_memory() for k in dev} if host_io else dev
+    r = rs.contiguous().pin_memory() if host_io else rs.cuda()
+    x = torch.zeros_like(r).pin_memory() if host_io else torch.zeros_like(r)
+    server.submit(1, S, N, nb, nr, src["D"], src["E"], src["C"], src["R"], r, x, host_io=host_io)
+    (c,) = server.drain()
+    server.close()
+    assert [bool((x[j].cpu() == ref[j]).all()) for j in range(3)] == [True] * 3
+    assert c["iters"] == [i["iters"] for i in infos]
+    assert c["backward_error"] == [i["backward_error"] for i in infos]
