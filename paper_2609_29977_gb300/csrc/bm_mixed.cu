@@ -33,6 +33,7 @@
 
 #include "bm_coupling.cuh"
 #include "bm_mixed.cuh"
+#include "bm_solve_chain.cuh"
 
 namespace bm {
 namespace {
@@ -73,6 +74,32 @@ __global__ void __launch_bounds__(256) k_mixed_bwd(MixedState m, double *x, int 
   pdl_wait();
   if (ir_done(m.ctl)) return;
   bwd_tail<NB>(m, x, ir_iter(m.ctl, iter), blockIdx.x / CS, (int)cluster_rank(), CS, sX);
+}
+
+// The same two kernels for few tails (chain_applies): one CTA per tail.
+template <int NB>
+__global__ void __launch_bounds__(256, ChainCfg<NB>::CTAS) k_mixed_fwd_chain(MixedState m,
+                                                                             const double *__restrict__ r, double *x,
+                                                                             int iter,
+                                                                             cudaGraphConditionalHandle cond) {
+  extern __shared__ __align__(16) double sV[];   // the tail's vectors, then the root step
+  __shared__ float sY[MCfg<NB>::TEAMS][NB];
+  pdl_wait();
+  if (iter < 0 && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(cond, 0u);
+  if (ir_done(m.ctl)) return;
+  const int it = ir_iter(m.ctl, iter);
+  const double *rhs = it == 0 ? r : m.rho;
+  fwd_tail_chain<NB>(m, rhs, blockIdx.x, (float *)sV, sY);
+  if (last_cta(&m.tickets[2], gridDim.x)) root_step<NB>(m, rhs, x, it, sV, coupled(m) ? xt_blocks(m.S, m.N, NB, m.nr) : m.S);
+}
+
+template <int NB>
+__global__ void __launch_bounds__(256, ChainCfg<NB>::CTAS) k_mixed_bwd_chain(MixedState m, double *x, int iter) {
+  extern __shared__ __align__(16) double sV[];
+  __shared__ float sX[MCfg<NB>::TEAMS][NB];
+  pdl_wait();
+  if (ir_done(m.ctl)) return;
+  bwd_tail_chain<NB>(m, x, ir_iter(m.ctl, iter), blockIdx.x, (float *)sV, sX);
 }
 
 // rho = r - K x in FP64 and the componentwise backward error of the
@@ -345,9 +372,15 @@ template <int NB>
 void launch_iteration(const MixedState &m, const double *r, double *x, int iter, int max_iter, double tol,
                       cudaStream_t st, cudaGraphConditionalHandle cond, bool pdl) {
   const int CS = pick_cluster(m.S);
-  const unsigned grid = (unsigned)(m.S * CS);
-  launch_cluster(k_mixed_fwd<NB>, grid, 256, CS, pdl, st, m, r, x, iter, CS, cond);
-  launch_cluster(k_mixed_bwd<NB>, grid, 256, CS, pdl, st, m, x, iter, CS);
+  if (chain_applies<NB>(m.S, m.N, CS)) {
+    const size_t vec = (size_t)m.N * NB * sizeof(float), root = ((size_t)m.nr * m.nr + m.nr) * sizeof(double);
+    launch_plain(k_mixed_fwd_chain<NB>, (unsigned)m.S, 256, vec > root ? vec : root, pdl, st, m, r, x, iter, cond);
+    launch_plain(k_mixed_bwd_chain<NB>, (unsigned)m.S, 256, vec, pdl, st, m, x, iter);
+  } else {
+    const unsigned grid = (unsigned)(m.S * CS);
+    launch_cluster(k_mixed_fwd<NB>, grid, 256, CS, pdl, st, m, r, x, iter, CS, cond);
+    launch_cluster(k_mixed_bwd<NB>, grid, 256, CS, pdl, st, m, x, iter, CS);
+  }
   const int blocks = xt_blocks(m.S, m.N, NB, m.nr);
   launch_plain(k_mixed_residual<NB>, (unsigned)blocks, 256, FFCfg<NB>::bytes, pdl, st, m, r, (const double *)x, iter, max_iter, tol,
                cond);
@@ -505,7 +538,11 @@ cudaError_t mixed_prepare(int nb, int nr) {
   if (e == cudaSuccess)                                                                                       \
     e = cudaFuncSetAttribute(k_mixed_residual<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);    \
   if (e == cudaSuccess)                                                                                       \
-    e = cudaFuncSetAttribute(k_residual_out<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
+    e = cudaFuncSetAttribute(k_residual_out<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);      \
+  if (e == cudaSuccess)                                                                                       \
+    e = cudaFuncSetAttribute(k_mixed_fwd_chain<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);   \
+  if (e == cudaSuccess)                                                                                       \
+    e = cudaFuncSetAttribute(k_mixed_bwd_chain<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
   BM_TAIL_NB_LIST(X)
 #undef X
   if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
@@ -637,6 +674,7 @@ void retry_root(const MixedState &m, cudaStream_t st) {
 }
 }  // namespace
 
+// unroll, resume: directly launched only, see the declaration in bm_api.cu.
 cudaError_t mixed_launch_solve(MixedState *m, const double *r, double *x, int max_refine, double tol,
                                cudaStream_t st, cudaStream_t body_st, cudaStream_t if_st, cudaStream_t body2_st,
                                bool body_pdl, int unroll, bool resume) {
@@ -674,7 +712,6 @@ cudaError_t mixed_launch_solve(MixedState *m, const double *r, double *x, int ma
   case n:                                                        \
     launch_iteration<n>(*m, r, x, it, max_refine, tol, st, 0, true); \
     break;
-// unroll, resume: directly launched only, see the declaration in bm_api.cu.
       BM_TAIL_NB_LIST(X)
 #undef X
     }
