@@ -447,6 +447,7 @@ size_t f64_factor_smem(int nb, int nr) {
 }
 
 bool f64_cluster_solve_supported(int nb);
+cudaError_t f64_solve_prepare();
 void f64_cluster_launch_solve(const F64View &v, const double *r, double *x, cudaStream_t st);
 
 // The dynamic shared-memory limit is a per-kernel attribute shared by every
@@ -478,6 +479,7 @@ cudaError_t f64_prepare(int nb, int nr) {
                            (int)(((size_t)nr * nr + nr) * sizeof(double)));
   if (e != cudaSuccess) return e;
   e = tail_factor_prepare();
+  if (e == cudaSuccess) e = f64_solve_prepare();
   if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;   // only once everything was set
   return e;
 }

@@ -1,0 +1,64 @@
+"""The substitutions of few tails (one CTA per tail, vectors in shared memory)
+against the cluster kernels, bit for bit.
+
+FP64: a system of the largest S that takes the first form, and the same system
+with one more tail, whose coupling block is zero, which takes the second. That
+tail adds exact zeros to the root, so every other component of x has to be
+the same. Mixed precision: the batched form, whose substitutions are those of
+the cluster kernels (another tail would move the root's residual terms to
+other partial sums).
+"""
+import pytest
+import torch
+
+import bmgen
+
+pytestmark = pytest.mark.gpu
+
+
+def _solve(bm, d, S):
+    solver = bm.BranchKKTSolver(S, d["N"], d["nb"], d["nr"])
+    solver.factor(d["D"], d["E"], d["C"], d["R"])
+    x = solver.solve(d["r"])
+    torch.cuda.synchronize()
+    assert solver.query()["status"] == 0
+    solver.close()
+    return x
+
+
+def _system(S, N, nb):
+    w = bmgen.Workload("f", S, N, nb, max(1, nb // 3), workload_id=95, barrier=(-2.0, 2.0), shared_A=True)
+    return bmgen.generate(w, seed=11, device="cuda")
+
+
+# S the last of the few-tails form; N = 1, at and beside powers of two, and
+# more positions than one round of a CTA's teams
+@pytest.mark.parametrize("S,N,nb", [(304, 1, 4), (304, 9, 4), (304, 6, 3), (304, 40, 12), (304, 33, 16), (152, 17, 24),
+                                    (152, 50, 24)])
+def test_few_tails_form_gives_the_cluster_kernels_bits(S, N, nb):
+    import paper_2609_29977_gb300 as bm
+    d = _system(S, N, nb)
+    n, nr = S * N * nb, d["nr"]
+    more = {k: torch.cat([d[k], d[k][:1]]) for k in ("D", "E", "C")}
+    more["C"][S:] = 0.0
+    more.update(R=d["R"], N=N, nb=nb, nr=nr, r=torch.cat([d["r"][:n], d["r"][:N * nb], d["r"][n:]]))
+    a, b = _solve(bm, d, S), _solve(bm, more, S + 1)
+    assert torch.equal(a[:n], b[:n]) and torch.equal(a[n:], b[-nr:])
+
+
+@pytest.mark.parametrize("S,N,nb", [(304, 1, 4), (304, 2, 4), (304, 8, 6), (304, 33, 12), (304, 40, 24), (152, 13, 48)])
+def test_few_tails_form_gives_the_batched_forms_bits(S, N, nb, tmp_path, monkeypatch):
+    import paper_2609_29977_gb300 as bm
+    monkeypatch.setenv("BM_AUTOTUNE_CACHE", str(tmp_path / "tune.json"))
+    d = _system(S, N, nb)
+    tol = 1e-12   # FP64 residuals, as in the batched form
+    solver = bm.BranchKKTSolver(S, N, nb, d["nr"], precision=bm.BM_PREC_FP32_IR, tol=tol)
+    solver.factor(d["D"], d["E"], d["C"], d["R"])
+    x, info = solver.solve(d["r"]), solver.query()
+    solver.close()
+    batch = bm.BranchKKTBatch([(S, N, nb, d["nr"])], tol=tol)
+    batch.factor([d["D"]], [d["E"]], [d["C"]], [d["R"]])
+    (xb,), (ib,) = batch.solve([d["r"]]), batch.query()
+    batch.close()
+    assert info["status"] == ib["status"] == 0 and info["iters"] == ib["iters"] >= 1
+    assert torch.equal(x, xb)
