@@ -123,9 +123,7 @@ __global__ void __launch_bounds__(256, FFCfg<NB>::STAGED ? 3 : 5) k_mixed_residu
   const bool ffr = m.ffres && __ldcg(&m.status->ffbad) == 0;
   float om = 0.0f;
   if (ffr) {
-    const int warp = threadIdx.x >> 5;
-    for (long e0 = (long)blockIdx.x * blockDim.x + 32 * warp; e0 < nrow; e0 += (long)gridDim.x * blockDim.x)
-      om = fmaxf(om, residual_rows_ff<NB>(m, r, x, e0, nrow, sE + warp * 2 * FFCfg<NB>::PLANE));
+    om = residual_ff<NB>(m, r, x, sE);
   } else {
     for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < nrow; e += (long)gridDim.x * blockDim.x) {
       const long br = e / NB;
@@ -274,9 +272,7 @@ __global__ void __launch_bounds__(256) k_residual_out(MixedState m, const double
   const long nrow = (long)m.S * m.N * NB;
   const bool ffr = m.ffres && __ldcg(&m.status->ffbad) == 0;
   if (ffr) {
-    const int warp = threadIdx.x >> 5;
-    for (long e0 = (long)blockIdx.x * blockDim.x + 32 * warp; e0 < nrow; e0 += (long)gridDim.x * blockDim.x)
-      residual_rows_ff<NB>(m, r, x, e0, nrow, sE + warp * 2 * FFCfg<NB>::PLANE);
+    residual_ff<NB>(m, r, x, sE);
   } else {
     for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < nrow; e += (long)gridDim.x * blockDim.x) {
       const long br = e / NB;

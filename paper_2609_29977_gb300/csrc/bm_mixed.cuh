@@ -579,12 +579,13 @@ constexpr double kFFBeta = 4e-12;
 constexpr double kFFMinTol = 1e-11;
 
 // NB terms: K's entries at kh/kl[t * STRIDE] (global or shared memory), x's
-// contiguous; groups of four per load where both allow it.
-template <int NB, int STRIDE>
+// contiguous; four per load where rows allow it (x beside a column of K:
+// only where WIDE asks for it, the narrow kernels lose registers by it).
+template <int NB, int STRIDE, bool WIDE = false>
 __device__ __forceinline__ void ff_block(double &acc, float &w, const float *__restrict__ kh,
                                          const float *__restrict__ kl, const float *__restrict__ xh,
                                          const float *__restrict__ xl) {
-  constexpr bool V4 = NB % 4 == 0;
+  constexpr bool V4 = NB % 4 == 0 && (STRIDE == 1 || WIDE);
 #pragma unroll
   for (int j0 = 0; j0 < NB; j0 += 8) {
     constexpr int CH = 8;
@@ -641,9 +642,49 @@ __device__ __forceinline__ void ff_block(double &acc, float &w, const float *__r
   }
 }
 
+// Row i of block row (s, k) of the residual in float-float; as
+// residual_row, but (|K||x|)_i from the hi parts (scaled down by 2^-22 to
+// cover their rounding, so omega is never understated).
+template <int NB>
+__device__ __forceinline__ float residual_row_ff(const MixedState &m, const double *__restrict__ r,
+                                                 const double *__restrict__ x, int s, int k, int i) {
+  constexpr int NB2 = NB * NB;
+  const int N = m.N, nr = m.nr;
+  const size_t n0 = (size_t)m.S * N * NB;
+  const long br = (long)s * N + k;
+  const size_t off = (size_t)br * NB;
+  double acc = 0.0;
+  float w = 0.0f;
+  {
+    const size_t kb = (size_t)br * NB2 + (size_t)i * NB;
+    ff_block<NB, 1>(acc, w, m.Kdh + kb, m.Kdl + kb, m.xh + off, m.xl + off);
+  }
+  if (k > 0) {   // block (k, k-1) = E_k: row i
+    const size_t eb = ((size_t)s * (N - 1) + (k - 1)) * NB2 + (size_t)i * NB;
+    ff_block<NB, 1>(acc, w, m.Keh + eb, m.Kel + eb, m.xh + off - NB, m.xl + off - NB);
+  }
+  if (k + 1 < N) {   // block (k, k+1) = E_{k+1}^T: column i of E_{k+1}
+    const size_t eb = ((size_t)s * (N - 1) + k) * NB2 + i;
+    ff_block<NB, NB>(acc, w, m.Keh + eb, m.Kel + eb, m.xh + off + NB, m.xl + off + NB);
+  }
+  const double ri = r[off + i];
+  double rho = ri - acc;
+  w = __fadd_rd(__fmul_rd(w, __int_as_float(0x3f7ffffc)), abs_f32_approx(ri));   // 1 - 2^-22
+  if (k == 0) {   // block (1, root) = C_s^T, in FP64
+    const double *Cs = m.C + (size_t)s * nr * NB + i;
+    const double *x0 = x + n0;
+    for (int j = 0; j < nr; ++j) {
+      rho = fma(-Cs[j * NB], x0[j], rho);
+      w = fmaf(abs_f32_approx(Cs[j * NB]), abs_f32_approx(x0[j]), w);
+    }
+  }
+  m.rho[off + i] = rho;
+  return omega_of(rho, w);
+}
+
 // Shared memory of the float-float residual for wide blocks: per warp 32 rows
 // of E (hi and lo planes) of CW columns at a time, row stride an odd number of
-// 16-byte groups. Smaller blocks read the rows directly (below).
+// 16-byte groups. Smaller blocks read the rows directly (residual_row_ff).
 template <int NB>
 struct FFCfg {
   static constexpr bool STAGED = NB > 32;
@@ -653,13 +694,12 @@ struct FFCfg {
   static constexpr size_t bytes = STAGED ? (size_t)8 * 2 * PLANE * sizeof(float) : 0;   // eight warps
 };
 
-// 32 consecutive rows e0 + lane of the residual over all tails in
-// float-float (row e = block row (s, k), row i in it); as residual_row, but
-// (|K||x|)_i from the hi parts (scaled down by 2^-22 to cover their rounding,
-// so omega is never understated). Returns the lane's omega (0 beyond nrow).
+// 32 consecutive rows e0 + lane of the residual over all tails (row e = block
+// row (s, k), row i in it), wide blocks; the same operations as
+// residual_row_ff. Returns the lane's omega (0 beyond nrow).
 // buf: 2 * FFCfg<NB>::PLANE floats of the warp.
 //
-// For wide blocks D's row i is read as column i of the symmetric block,
+// D's row i is read as column i of the symmetric block,
 // contiguous over the lanes (the same values in the same order), and the
 // rows of E_k that 32 consecutive rows need, contiguous in memory, arrive
 // through shared memory by asynchronous copies behind D's part: nb = 48,
@@ -693,35 +733,25 @@ __device__ __forceinline__ float residual_rows_ff(const MixedState &m, const dou
       }
     }
   };
-  if constexpr (FFCfg<NB>::STAGED) stage_e(0);
+  stage_e(0);
   double acc = 0.0;
   float w = 0.0f;
   if (ok) {
-    if constexpr (FFCfg<NB>::STAGED) {
-      const size_t kb = (size_t)br * NB2 + i;   // column i of the symmetric block
-      ff_block<NB, NB>(acc, w, m.Kdh + kb, m.Kdl + kb, m.xh + off, m.xl + off);
-    } else {
-      const size_t kb = (size_t)br * NB2 + (size_t)i * NB;
-      ff_block<NB, 1>(acc, w, m.Kdh + kb, m.Kdl + kb, m.xh + off, m.xl + off);
-    }
+    const size_t kb = (size_t)br * NB2 + i;   // column i of the symmetric block
+    ff_block<NB, NB, true>(acc, w, m.Kdh + kb, m.Kdl + kb, m.xh + off, m.xl + off);
   }
-  if constexpr (FFCfg<NB>::STAGED) {   // block (k, k-1) = E_k: row i
 #pragma unroll
-    for (int c0 = 0; c0 < NB; c0 += CW) {
-      rows::cp_async_wait();
-      __syncwarp();
-      if (erow >= 0)
-        ff_block<CW, 1>(acc, w, bh + lane * LD, bl + lane * LD, m.xh + off - NB + c0, m.xl + off - NB + c0);
-      __syncwarp();
-      if (c0 + CW < NB) stage_e(c0 + CW);
-    }
-  } else if (erow >= 0) {
-    ff_block<NB, 1>(acc, w, m.Keh + erow * NB, m.Kel + erow * NB, m.xh + off - NB, m.xl + off - NB);
+  for (int c0 = 0; c0 < NB; c0 += CW) {   // block (k, k-1) = E_k: row i
+    rows::cp_async_wait();
+    __syncwarp();
+    if (erow >= 0) ff_block<CW, 1>(acc, w, bh + lane * LD, bl + lane * LD, m.xh + off - NB + c0, m.xl + off - NB + c0);
+    __syncwarp();
+    if (c0 + CW < NB) stage_e(c0 + CW);
   }
   if (!ok) return 0.0f;
   if (k + 1 < N) {   // block (k, k+1) = E_{k+1}^T: column i of E_{k+1}
     const size_t eb = ((size_t)s * (N - 1) + k) * NB2 + i;
-    ff_block<NB, NB>(acc, w, m.Keh + eb, m.Kel + eb, m.xh + off + NB, m.xl + off + NB);
+    ff_block<NB, NB, true>(acc, w, m.Keh + eb, m.Kel + eb, m.xh + off + NB, m.xl + off + NB);
   }
   const double ri = r[off + i];
   double rho = ri - acc;
@@ -736,6 +766,28 @@ __device__ __forceinline__ float residual_rows_ff(const MixedState &m, const dou
   }
   m.rho[off + i] = rho;
   return omega_of(rho, w);
+}
+
+// The calling thread's largest omega over its rows of the whole grid; buf:
+// the block's shared memory (FFCfg<NB>::bytes).
+template <int NB>
+__device__ __forceinline__ float residual_ff(const MixedState &m, const double *__restrict__ r,
+                                             const double *__restrict__ x, float *buf) {
+  const long nrow = (long)m.S * m.N * NB, step = (long)gridDim.x * blockDim.x;
+  float om = 0.0f;
+  if constexpr (FFCfg<NB>::STAGED) {
+    const int warp = threadIdx.x >> 5;
+    for (long e0 = (long)blockIdx.x * blockDim.x + 32 * warp; e0 < nrow; e0 += step)
+      om = fmaxf(om, residual_rows_ff<NB>(m, r, x, e0, nrow, buf + warp * 2 * FFCfg<NB>::PLANE));
+  } else {
+    for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < nrow; e += step) {
+      const long br = e / NB;
+      const int i = (int)(e - br * NB);
+      const int s = (int)(br / m.N), k = (int)(br - (long)s * m.N);
+      om = fmaxf(om, residual_row_ff<NB>(m, r, x, s, k, i));
+    }
+  }
+  return om;
 }
 
 // Folds a lane's omega into the warp and then into the system's wmax.

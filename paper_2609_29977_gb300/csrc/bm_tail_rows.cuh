@@ -645,9 +645,11 @@ __global__ void __launch_bounds__(128, 4) k_level_rows(TailView<T> v, int lvl) {
   pdl_trigger();
 }
 
-// Top levels lvl0..Lc-1 and x_1 of one tail per CTA (four teams).
+// Top levels lvl0..Lc-1 and x_1 of one tail per CTA (four teams). Four CTAs
+// per SM: left to itself the compiler takes 255 registers for nb = 24, two
+// CTAs fit and 512 tails need two waves (S = 512, N = 128: 154 -> 109 us).
 template <typename T, int NB>
-__global__ void __launch_bounds__(128) k_top_rows(TailView<T> v, int lvl0) {
+__global__ void __launch_bounds__(128, 4) k_top_rows(TailView<T> v, int lvl0) {
   constexpr int TS = Cfg<NB>::TS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int team = threadIdx.x / TS, lane = threadIdx.x % TS, teams = blockDim.x / TS;
