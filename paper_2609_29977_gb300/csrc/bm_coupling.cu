@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(XCfg<NB>::THREADS, XCfg<NB>::MINB) k_cx_fwd(Cx
   pdl_trigger();
 }
 
-template <int NB>
+template <int NB, bool PLANES>
 __global__ void __launch_bounds__(256, 4) k_cx_residual(CxView v) {
   pdl_wait();
   if (engaged(v)) {
@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(256, 4) k_cx_residual(CxView v) {
       const long br = e / NB;
       const int i = (int)(e - br * NB);
       const int s = (int)(br / v.N), k = (int)(br - (long)s * v.N);
-      residual_row_multi<NB>(v, s, k, i);
+      residual_row_multi<NB, PLANES>(v, s, k, i);
     }
   }
   pdl_trigger();
@@ -90,7 +90,7 @@ void launch_nb(const CxView &v, int *mark, cudaStream_t st) {
   const long rows = (long)v.S * v.N * NB;
   long blocks = (rows + 255) / 256;
   if (blocks > 152 * 8) blocks = 152 * 8;
-  launch_cx(k_cx_residual<NB>, (unsigned)blocks, 256u, 1, st, v);
+  launch_cx(v.Kdh ? k_cx_residual<NB, true> : k_cx_residual<NB, false>, (unsigned)blocks, 256u, 1, st, v);
   launch_cx(k_cx_fwd<NB>, grid, THR, CS, st, v, CS);
   launch_cx(k_cx_bwd<NB>, grid, THR, CS, st, v, 1, CS, (int *)nullptr);
 }

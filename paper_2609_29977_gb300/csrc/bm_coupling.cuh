@@ -38,6 +38,9 @@ struct CxView {
   int S, N, nr, ldc, Lc;
   const float *Ld, *Ll, *Lr, *invd;   // FP32 tail factor
   const double *D, *E, *C;            // FP64 inputs
+  // hi + lo planes of D (symmetric rows) and E where the handle keeps them
+  // for its float-float residuals (null otherwise)
+  const float *Kdh, *Kdl, *Keh, *Kel;
   float *Xa;   // [S][N][nb][ldc] X0, then the refined X (rounded to FP32)
   float *Yb;   // [S][N][nb][ldc] forward vectors, then the correction d
   float *Zr;   // [S][N][nb][ldc] residual P, then partial gathers in place
@@ -370,14 +373,18 @@ __device__ __forceinline__ void bwd_multi(const CxView &v, int s, int crank, int
 // P = C_i^T - K_i X0 for one row (tail s, natural stage k + 1, block row i)
 // and all ldc right-hand sides, exact to about 2^-46 relative to
 // |C^T| + |K| |X0|: every FP64 entry is split into hi + lo floats and the
-// products with the (exactly FP32) X0 are summed by Dot2.
-template <int NB>
+// products with the (exactly FP32) X0 are summed by Dot2. PLANES: the
+// entries' hi and lo parts are read from the planes that the float-float
+// residuals use (the same split, about 25 of the 110 instructions per entry
+// and eight columns otherwise): nb = 24, S = 512, N = 128: 538 -> 416 us.
+template <int NB, bool PLANES>
 __device__ __forceinline__ void residual_row_multi(const CxView &v, int s, int k, int i) {
   constexpr int NB2 = NB * NB;
   const int N = v.N, nr = v.nr, ldc = v.ldc;
   const size_t br = (size_t)s * N + k;
-  const double *Dk = v.D + br * NB2;
   const float *xk = v.Xa + br * NB * ldc;
+  const size_t el = ((size_t)s * (N - 1) + (k - 1)) * NB2 + i * NB;   // row i of E_k (k > 0)
+  const size_t er = ((size_t)s * (N - 1) + k) * NB2 + i;              // column i of E_{k+1} (k + 1 < N)
   for (int c0 = 0; c0 < ldc; c0 += RC) {
     float sh[RC], sl[RC];
 #pragma unroll
@@ -386,26 +393,51 @@ __device__ __forceinline__ void residual_row_multi(const CxView &v, int s, int k
       sl[c] = 0.0f;
       if (k == 0 && c0 + c < nr) ff::split_d(v.C[((size_t)s * nr + c0 + c) * NB + i], sh[c], sl[c]);
     }
-    auto block = [&](auto kij_of, const float *xb) {
+    auto entry = [&](float kh, float kl, const float *xr) {
+      const float4 a = *reinterpret_cast<const float4 *>(xr);
+      const float4 b = *reinterpret_cast<const float4 *>(xr + 4);
+      const float xv[RC] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+      for (int c = 0; c < RC; ++c) ff::dot2_step_split(sh[c], sl[c], -kh, -kl, xv[c]);
+    };
+    auto block = [&](auto kij_of, const float *xb) {   // FP64 entries
 #pragma unroll 4
       for (int j = 0; j < NB; ++j) {
         float kh, kl;
         ff::split_d(kij_of(j), kh, kl);
-        const float4 a = *reinterpret_cast<const float4 *>(xb + (size_t)j * ldc + c0);
-        const float4 b = *reinterpret_cast<const float4 *>(xb + (size_t)j * ldc + c0 + 4);
-        const float xv[RC] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-#pragma unroll
-        for (int c = 0; c < RC; ++c) ff::dot2_step_split(sh[c], sl[c], -kh, -kl, xv[c]);
+        entry(kh, kl, xb + (size_t)j * ldc + c0);
       }
     };
-    block([&](int j) { return j <= i ? Dk[i * NB + j] : Dk[j * NB + i]; }, xk);
-    if (k > 0) {   // block (k, k-1) = E_k
-      const double *Ek = v.E + ((size_t)s * (N - 1) + (k - 1)) * NB2 + i * NB;
-      block([&](int j) { return Ek[j]; }, xk - NB * ldc);
-    }
-    if (k + 1 < N) {   // block (k, k+1) = E_{k+1}^T
-      const double *Ek = v.E + ((size_t)s * (N - 1) + k) * NB2 + i;
-      block([&](int j) { return Ek[j * NB]; }, xk + NB * ldc);
+    auto row = [&](const float *ph, const float *pl, const float *xb) {   // a row of the planes
+      if constexpr (NB % 4 == 0) {
+#pragma unroll 1
+        for (int j = 0; j < NB; j += 4) {
+          const float4 h = *reinterpret_cast<const float4 *>(ph + j), l = *reinterpret_cast<const float4 *>(pl + j);
+          const float *xr = xb + (size_t)j * ldc + c0;
+          entry(h.x, l.x, xr);
+          entry(h.y, l.y, xr + ldc);
+          entry(h.z, l.z, xr + 2 * ldc);
+          entry(h.w, l.w, xr + 3 * ldc);
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < NB; ++j) entry(ph[j], pl[j], xb + (size_t)j * ldc + c0);
+      }
+    };
+    auto col = [&](const float *ph, const float *pl, const float *xb) {   // a column
+#pragma unroll 4
+      for (int j = 0; j < NB; ++j) entry(ph[j * NB], pl[j * NB], xb + (size_t)j * ldc + c0);
+    };
+    if constexpr (PLANES) {
+      const size_t d = br * NB2 + (size_t)i * NB;
+      row(v.Kdh + d, v.Kdl + d, xk);
+      if (k > 0) row(v.Keh + el, v.Kel + el, xk - NB * ldc);           // block (k, k-1) = E_k
+      if (k + 1 < N) col(v.Keh + er, v.Kel + er, xk + NB * ldc);       // block (k, k+1) = E_{k+1}^T
+    } else {
+      const double *Dk = v.D + br * NB2;
+      block([&](int j) { return j <= i ? Dk[i * NB + j] : Dk[j * NB + i]; }, xk);
+      if (k > 0) block([&](int j) { return v.E[el + j]; }, xk - NB * ldc);
+      if (k + 1 < N) block([&](int j) { return v.E[er + (size_t)j * NB]; }, xk + NB * ldc);
     }
     float *o = v.Zr + (br * NB + i) * ldc + c0;
     float r[RC];

@@ -610,6 +610,8 @@ static cx::CxView cx_view(const MixedState &m, int *on) {
   cv.S = m.S; cv.N = m.N; cv.nr = m.nr; cv.ldc = m.ldc; cv.Lc = m.Lc;
   cv.Ld = m.Ld; cv.Ll = m.Ll; cv.Lr = m.Lr; cv.invd = m.invd;
   cv.D = m.D; cv.E = m.E; cv.C = m.C;
+  cv.Kdh = m.ffres ? m.Kdh : nullptr;
+  cv.Kdl = m.Kdl; cv.Keh = m.Keh; cv.Kel = m.Kel;
   cv.Xa = m.Xa; cv.Yb = m.Yb; cv.Zr = m.Zr; cv.U = m.U;
   cv.on = on;
   return cv;
