@@ -196,10 +196,20 @@ __device__ __forceinline__ void block_out(float *__restrict__ g, const float *__
 // An FP64 input block, rounded to FP32, into shared memory: two doubles per
 // load, contiguous over the team, all loads before the first conversion (the
 // hardware rounding, see load_to_t). LOWER: only pairs that reach the lower triangle.
+// Single loads where the caller's array is not 16-byte aligned (a batch takes
+// pointers that the host does not see).
 template <int NB, int TS, bool LOWER, int LD = Cfg<NB>::LD>
 __device__ __forceinline__ void block_in_d(float *__restrict__ s, const double *__restrict__ g, int lane) {
   // 9 loads in flight per lane (all of a 24 x 24 block, half of a 48 x 48 one)
   constexpr int Q = NB * NB / 2, M = (Q + TS - 1) / TS, CH = M < 9 ? M : 9;
+  if ((reinterpret_cast<unsigned long long>(g) & 15) != 0) {
+#pragma unroll 1
+    for (int e = lane; e < NB * NB; e += TS) {
+      const int r = e / NB, c = e - r * NB;
+      if (!LOWER || c <= r) s[r * LD + c] = __double2float_rn(g[e]);
+    }
+    return;
+  }
 #pragma unroll
   for (int t0 = 0; t0 < M; t0 += CH) {
     double2 v[CH];

@@ -62,3 +62,29 @@ def test_few_tails_form_gives_the_batched_forms_bits(S, N, nb, tmp_path, monkeyp
     batch.close()
     assert info["status"] == ib["status"] == 0 and info["iters"] == ib["iters"] >= 1
     assert torch.equal(x, xb)
+
+
+# arrays eight bytes off a 16-byte boundary, which a batch has always taken
+@pytest.mark.parametrize("nb", [4, 6, 24, 48])
+def test_batch_takes_arrays_eight_bytes_off(nb, tmp_path, monkeypatch):
+    import paper_2609_29977_gb300 as bm
+    monkeypatch.setenv("BM_AUTOTUNE_CACHE", str(tmp_path / "tune.json"))
+    S, N = 3, 6
+    d = _system(S, N, nb)
+
+    def off(t):
+        buf = torch.empty(t.numel() + 1, dtype=t.dtype, device=t.device)
+        v = buf[1:].view(t.shape)
+        v.copy_(t)
+        assert v.data_ptr() % 16 == 8
+        return v
+
+    xs = []
+    for f in (lambda t: t, off):
+        batch = bm.BranchKKTBatch([(S, N, nb, d["nr"])])
+        batch.factor([f(d["D"])], [f(d["E"])], [f(d["C"])], [f(d["R"])])
+        (x,) = batch.solve([f(d["r"])])
+        assert batch.query()[0]["status"] == 0
+        batch.close()
+        xs.append(x)
+    assert torch.equal(*xs)
