@@ -21,10 +21,12 @@ __global__ void k_batch_reset(BInst *inst, int ninst) {
   inst[b].m.tickets[3] = 0u;
 }
 
-__global__ void __launch_bounds__(256) k_batch_fwd(const BInst *inst, const BTail *tails, const double *const *rp,
+constexpr int kSubFloats = SubCfg<48>::floats(256);   // the widest block's
+
+__global__ void __launch_bounds__(256, 3) k_batch_fwd(const BInst *inst, const BTail *tails, const double *const *rp,
                                                    double *const *xp, int iter) {
-  __shared__ __align__(16) float sbuf[256];
-  __shared__ double sR[64 * 64 + 128];
+  // the tail's part, then the root step
+  __shared__ __align__(16) double sbuf[kSubFloats / 2 > 64 * 64 + 128 ? kSubFloats / 2 : 64 * 64 + 128];
   const BTail t = tails[blockIdx.x];
   const BInst &I = inst[t.inst];
   pdl_wait();
@@ -33,15 +35,20 @@ __global__ void __launch_bounds__(256) k_batch_fwd(const BInst *inst, const BTai
   switch (I.nb) {
 #define X(n)                                                              \
   case n:                                                                 \
-    fwd_tail<n>(I.m, rhs, t.s, 0, 1, reinterpret_cast<float(*)[n]>(sbuf)); \
-    if (last_cta(&I.m.tickets[2], (unsigned)I.S)) root_step<n>(I.m, rhs, xp[t.inst], iter, sR, I.S); \
+    fwd_tail<n>(I.m, rhs, t.s, 0, 1, (float *)sbuf);                       \
+    if (last_cta(&I.m.tickets[2], (unsigned)I.S)) root_step<n>(I.m, rhs, xp[t.inst], iter, sbuf, I.S); \
     break;
     BM_BATCH_NB_LIST(X)
 #undef X
   }
 }
 
-__global__ void __launch_bounds__(256) k_batch_bwd(const BInst *inst, const BTail *tails, double *const *xp,
+// Wide blocks keep the teams of two warps here: the CTA's registers are set
+// by all block sizes (80 for three CTAs per SM), too few for the pair form's
+// loads in flight. Batch of 16 systems, per pass: 179 us, pair form 284 us
+// (262 us with two CTAs per SM). The forward form reads L_qq from shared
+// memory and gains: 290 -> 240 us.
+__global__ void __launch_bounds__(256, 3) k_batch_bwd(const BInst *inst, const BTail *tails, double *const *xp,
                                                    int iter) {
   __shared__ __align__(16) float sbuf[256];
   const BTail t = tails[blockIdx.x];
@@ -51,7 +58,7 @@ __global__ void __launch_bounds__(256) k_batch_bwd(const BInst *inst, const BTai
   switch (I.nb) {
 #define X(n)                                                                           \
   case n:                                                                              \
-    bwd_tail<n>(I.m, xp[t.inst], iter, t.s, 0, 1, reinterpret_cast<float(*)[n]>(sbuf)); \
+    bwd_tail<n, false>(I.m, xp[t.inst], iter, t.s, 0, 1, sbuf);                        \
     break;
     BM_BATCH_NB_LIST(X)
 #undef X

@@ -54,26 +54,27 @@ __host__ __device__ inline int xt_blocks(int S, int N, int nb, int nr) {
 // loop, whose iteration index is read from the control block and whose
 // condition handle is cond.
 template <int NB>
-__global__ void __launch_bounds__(256) k_mixed_fwd(MixedState m, const double *__restrict__ r, double *x, int iter,
+__global__ void __launch_bounds__(SubCfg<NB>::THREADS, 4) k_mixed_fwd(MixedState m, const double *__restrict__ r, double *x, int iter,
                                                     int CS, cudaGraphConditionalHandle cond) {
-  __shared__ float sY[MCfg<NB>::TEAMS][NB];
-  __shared__ double sR[64 * 64 + 64 + 64];
+  // the tail's part, then the root step
+  constexpr int F = SubCfg<NB>::floats(SubCfg<NB>::THREADS) / 2, R = 64 * 64 + 64 + 64;
+  __shared__ __align__(16) double sbuf[F > R ? F : R];
   pdl_wait();
   // the loop stops after this iteration unless its stopping test says otherwise
   if (iter < 0 && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(cond, 0u);
   if (ir_done(m.ctl)) return;
   const int it = ir_iter(m.ctl, iter);
   const double *rhs = it == 0 ? r : m.rho;
-  fwd_tail<NB>(m, rhs, blockIdx.x / CS, (int)cluster_rank(), CS, sY);
-  if (last_cta(&m.tickets[2], gridDim.x)) root_step<NB>(m, rhs, x, it, sR, coupled(m) ? xt_blocks(m.S, m.N, NB, m.nr) : m.S);
+  fwd_tail<NB>(m, rhs, blockIdx.x / CS, (int)cluster_rank(), CS, (float *)sbuf);
+  if (last_cta(&m.tickets[2], gridDim.x)) root_step<NB>(m, rhs, x, it, sbuf, coupled(m) ? xt_blocks(m.S, m.N, NB, m.nr) : m.S);
 }
 
 template <int NB>
-__global__ void __launch_bounds__(256) k_mixed_bwd(MixedState m, double *x, int iter, int CS) {
-  __shared__ float sX[MCfg<NB>::TEAMS][NB];
+__global__ void __launch_bounds__(SubCfg<NB>::THREADS, 4) k_mixed_bwd(MixedState m, double *x, int iter, int CS) {
+  __shared__ __align__(16) float sbuf[SubCfg<NB>::floats(SubCfg<NB>::THREADS)];
   pdl_wait();
   if (ir_done(m.ctl)) return;
-  bwd_tail<NB>(m, x, ir_iter(m.ctl, iter), blockIdx.x / CS, (int)cluster_rank(), CS, sX);
+  bwd_tail<NB>(m, x, ir_iter(m.ctl, iter), blockIdx.x / CS, (int)cluster_rank(), CS, sbuf);
 }
 
 // The same two kernels for few tails (chain_applies): one CTA per tail.
@@ -407,8 +408,8 @@ void launch_iteration(const MixedState &m, const double *r, double *x, int iter,
     launch_plain(k_mixed_bwd_chain<NB>, (unsigned)m.S, 256, vec, pdl, st, m, x, iter);
   } else {
     const unsigned grid = (unsigned)(m.S * CS);
-    launch_cluster(k_mixed_fwd<NB>, grid, 256, CS, pdl, st, m, r, x, iter, CS, cond);
-    launch_cluster(k_mixed_bwd<NB>, grid, 256, CS, pdl, st, m, x, iter, CS);
+    launch_cluster(k_mixed_fwd<NB>, grid, SubCfg<NB>::THREADS, CS, pdl, st, m, r, x, iter, CS, cond);
+    launch_cluster(k_mixed_bwd<NB>, grid, SubCfg<NB>::THREADS, CS, pdl, st, m, x, iter, CS);
   }
   const int blocks = xt_blocks(m.S, m.N, NB, m.nr);
   launch_plain(k_mixed_residual<NB>, (unsigned)blocks, 256, FFCfg<NB>::bytes, pdl, st, m, r, (const double *)x, iter, max_iter, tol,

@@ -86,6 +86,23 @@ struct MCfg {
   static constexpr int TEAMS = THREADS / TS;
 };
 
+// The substitutions of one tail by one CTA (or cluster): teams of TS threads,
+// one row per thread, up to nb = 32; above, one warp per position with rows i
+// and i + 32 on lane i and the position's L_qq in shared memory.
+template <int NB>
+struct SubCfg {
+  static constexpr bool PAIR = NB > 32;
+  static constexpr int THREADS = PAIR ? 128 : 256;
+  // row i of a lower triangle packed in groups of four floats, i / 4 + 1 groups each
+  __host__ __device__ static constexpr int row(int i) {
+    const int a = i >> 2;
+    return 4 * ((a + 1) * (2 * a + (i & 3)));
+  }
+  static constexpr int BLK = NB / 4 * (NB / 4 + 1) * 2 * 4;   // floats of one packed triangle
+  // floats of shared memory of a CTA of `threads`
+  static constexpr int floats(int threads) { return PAIR ? threads / 32 * BLK : threads; }
+};
+
 __device__ __forceinline__ bool ir_done(const IRCtl *ctl) {
   return *((volatile const int *)&ctl->converged) != 0;
 }
@@ -231,67 +248,241 @@ __device__ __forceinline__ void xt_grid(const MixedState &m, const double *__res
   }
 }
 
+// Substitutions of wide blocks (SubCfg::PAIR). A team of two warps would pay a
+// named barrier per column of L_qq (nb = 48: 9 of 27 stall cycles per
+// instruction) and hold half as many positions in flight per SM. A warp with
+// two rows per lane broadcasts by shuffles; L_qq arrives in shared memory by
+// asynchronous copies behind the gather, its lower triangle only, and leaves
+// the registers to the gather's loads. CTAs of 128 threads, four per SM, so
+// that 608 tails are resident at once. Every row's operations and their order
+// are those of the narrow form. S = 512, N = 256,
+// nb = 48: forward 1175 -> 793 us, backward 1045 -> 660 us per pass.
+template <int NB>
+__device__ __forceinline__ void pair_stage(float *buf, const float *__restrict__ L) {
+  constexpr int Q = NB / 4;
+  const int lane = threadIdx.x & 31;
+  __syncwarp();   // the last position's reads are done
+#pragma unroll
+  for (int u = 0; u < (NB * Q + 31) / 32; ++u) {
+    const int t = lane + 32 * u, row = t / Q, c = 4 * (t - row * Q);
+    if (row < NB && c <= row) rows::cp_async16(buf + SubCfg<NB>::row(row) + c, L + row * NB + c);
+  }
+}
+
+// (z0, z1) -= rows i and i + 32 of a block times y (k in increasing order)
+template <int NB>
+__device__ __forceinline__ void pair_row_dot(const float *__restrict__ L0, const float *__restrict__ L1, bool two,
+                                             const float *y, float &z0, float &z1) {
+  const float4 *y4 = reinterpret_cast<const float4 *>(y);
+  const float4 *a4 = reinterpret_cast<const float4 *>(L0), *b4 = reinterpret_cast<const float4 *>(L1);
+#pragma unroll
+  for (int g = 0; g < NB / 4; ++g) {
+    const float4 v = __ldcg(y4 + g), a = a4[g];
+    float4 b = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (two) b = b4[g];
+    z0 = fmaf(-a.x, v.x, z0);
+    z0 = fmaf(-a.y, v.y, z0);
+    z0 = fmaf(-a.z, v.z, z0);
+    z0 = fmaf(-a.w, v.w, z0);
+    z1 = fmaf(-b.x, v.x, z1);
+    z1 = fmaf(-b.y, v.y, z1);
+    z1 = fmaf(-b.z, v.z, z1);
+    z1 = fmaf(-b.w, v.w, z1);
+  }
+}
+template <int NB>
+__device__ __forceinline__ void pair_col_dot(const float *__restrict__ L, bool two, const float *y, float &z0,
+                                             float &z1) {
+  const float4 *y4 = reinterpret_cast<const float4 *>(y);
+#pragma unroll
+  for (int g = 0; g < NB / 4; ++g) {
+    const float4 v4 = __ldcg(y4 + g);
+    const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float *r = L + (4 * g + u) * NB;
+      z0 = fmaf(-r[0], v[u], z0);
+      z1 = fmaf(-(two ? r[32] : 0.0f), v[u], z1);
+    }
+  }
+}
+
+template <int NB>
+__device__ __forceinline__ void fwd_tail_pair(const MixedState &m, const double *__restrict__ rhs, int s, int crank,
+                                              int CS, float *sbuf) {
+  constexpr int NB2 = NB * NB;
+  static_assert(NB % 4 == 0 && NB <= 64, "two rows per lane, read four entries at a time");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, teams = blockDim.x >> 5;
+  const bool two = lane + 32 < NB;
+  const int i0 = lane, i1 = two ? lane + 32 : lane;
+  const int N = m.N, Lc = m.Lc;
+  const size_t sb = (size_t)s * N;
+  float *buf = sbuf + warp * SubCfg<NB>::BLK;
+  const bool xmode = coupled(m);
+  for (int lvl = 0; lvl <= Lc; ++lvl) {
+    const bool lastlvl = lvl == Lc;
+    const int ntask = lastlvl ? 1 : (lvl == 0 ? N / 2 : ((N - 1) >> lvl) + 1);
+    for (int t = crank * teams + warp; t < ntask; t += CS * teams) {
+      int q;
+      if (lastlvl) q = N;
+      else if (lvl == 0) q = 2 * t + 1;
+      else q = t < ((N - 1) >> lvl) ? (t + 1) << lvl : N;
+      const bool elim = lastlvl || (q < N && ctz32(q) == lvl);
+      const size_t pos = sb + (N - q), zoff = pos * NB;
+      float inv0 = 0.0f, inv1 = 0.0f;
+      if (elim) {
+        pair_stage<NB>(buf, m.Ld + pos * NB2);
+        inv0 = m.invd[zoff + i0];
+        inv1 = m.invd[zoff + i1];
+      }
+      float z0, z1;
+      if (lvl <= 1) {
+        z0 = __double2float_rn(rhs[zoff + i0]);
+        z1 = __double2float_rn(rhs[zoff + i1]);
+      } else {
+        z0 = __ldcg(m.zt + zoff + i0);
+        z1 = __ldcg(m.zt + zoff + i1);
+      }
+      if (lvl >= 1) {
+        const int h = 1 << (lvl - 1);
+        int pl = 0, pr = 0;
+        if (q < N) {
+          pl = q - h;
+          if (q + h <= N - 1) pr = q + h;
+        } else {
+          const int mm = ((N - 1) >> (lvl - 1)) << (lvl - 1);
+          if (ctz32(mm) == lvl - 1) pl = mm;
+        }
+        if (pl) {
+          const float *L = m.Lr + (sb + (N - pl)) * NB2;
+          pair_row_dot<NB>(L + i0 * NB, L + i1 * NB, two, m.y + (sb + (N - pl)) * NB, z0, z1);
+        }
+        if (pr) {
+          const float *L = m.Ll + (sb + (N - pr)) * NB2;
+          pair_row_dot<NB>(L + i0 * NB, L + i1 * NB, two, m.y + (sb + (N - pr)) * NB, z0, z1);
+        }
+      }
+      if (!elim) {
+        m.zt[zoff + i0] = z0;
+        if (two) m.zt[zoff + i1] = z1;
+        continue;
+      }
+      rows::cp_async_wait();
+      __syncwarp();
+      const float4 *L0 = reinterpret_cast<const float4 *>(buf + SubCfg<NB>::row(i0));
+      const float4 *L1 = reinterpret_cast<const float4 *>(buf + SubCfg<NB>::row(i1));
+#pragma unroll
+      for (int g = 0; g < NB / 4; ++g) {
+        float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        float4 b = a;
+        if (4 * g < 32 && 4 * g <= i0) a = L0[g];
+        if (4 * g <= i1) b = L1[g];
+        const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int j = 4 * g + u;
+          float yj;
+          if (j < 32) {
+            if (i0 == j) z0 *= inv0;
+            yj = __shfl_sync(0xffffffffu, z0, j);
+            if (i0 > j) z0 = fmaf(-av[u], yj, z0);
+            z1 = fmaf(-bv[u], yj, z1);
+          } else {
+            if (lane == j - 32) z1 *= inv1;
+            yj = __shfl_sync(0xffffffffu, z1, j - 32);
+            if (lane > j - 32) z1 = fmaf(-bv[u], yj, z1);
+          }
+        }
+      }
+      m.y[zoff + i0] = z0;
+      if (two) m.y[zoff + i1] = z1;
+      if (lastlvl && !xmode) {
+        __syncwarp();
+        buf[i0] = z0;
+        if (two) buf[i1] = z1;
+        __syncwarp();
+        const int nr = m.nr;
+        const double *Fs = m.F + (size_t)s * nr * NB;
+        for (int c = lane; c < nr; c += 32) {
+          double acc = 0.0;
+#pragma unroll
+          for (int k = 0; k < NB; ++k) acc = fma(Fs[c * NB + k], f2d_exact(buf[k]), acc);
+          m.tb[(size_t)s * nr + c] = acc;
+        }
+      }
+    }
+    if (CS > 1)
+      cluster_sync();
+    else
+      __syncthreads();
+  }
+}
+
 // Forward substitution of one tail in FP32 (all levels, then x_1 and
 // t_i = F_{i,1} y_1 in FP64); the last CTA of the grid does the root step
 // of Alg. 2 in FP64 and stores the root correction d_0 (and x_0 += d_0).
 template <int NB>
 __device__ __forceinline__ void fwd_tail(const MixedState &m, const double *__restrict__ rhs, int s, int crank,
-                                         int CS, float (*sY)[NB]) {
-  constexpr int TS = MCfg<NB>::TS, TEAMS = MCfg<NB>::TEAMS, NB2 = NB * NB;
-  const Team<TS> tm;
-  const int N = m.N, Lc = m.Lc;
-  const size_t sb = (size_t)s * N;
-  const int i = tm.lane;
-  const bool xmode = coupled(m);
-  for (int lvl = 0; lvl <= Lc; ++lvl) {
-    const bool lastlvl = lvl == Lc;
-    const int ntask = lastlvl ? 1 : (lvl == 0 ? N / 2 : ((N - 1) >> lvl) + 1);
-    for (int t = crank * TEAMS + tm.id; t < ntask; t += CS * TEAMS) {
-      int q;
-      if (lastlvl) q = N;
-      else if (lvl == 0) q = 2 * t + 1;
-      else {
-        const int cnt = (N - 1) >> lvl;
-        q = t < cnt ? (t + 1) << lvl : N;
-      }
-      const bool elim = lastlvl || (q < N && ctz32(q) == lvl);
-      const size_t zoff = (sb + (N - q)) * NB;
-      // row i of L_qq and 1/L_ii: for NB <= 16 loaded first, so that they
-      // share the gather's memory round trip (in bounds for every q); for
-      // larger blocks after it (loaded first they slowed the nb = 48 solve)
-      constexpr bool kEarly = NB <= 16;
-      float Lrow[NB];
-      float inv = 0.0f;
-      if constexpr (kEarly) {
-        load_row<NB>(Lrow, m.Ld + (sb + (N - q)) * NB2 + (i < NB ? i : 0) * NB);
-        inv = i < NB ? m.invd[zoff + i] : 0.0f;
-      }
-      float z = 0.0f;
-      if (i < NB) {
-        z = (lvl <= 1) ? __double2float_rn(rhs[zoff + i]) : __ldcg(m.zt + zoff + i);
-        if (lvl >= 1) {
-          const int h = 1 << (lvl - 1);
-          int pl = 0, pr = 0;
-          if (q < N) {
-            pl = q - h;
-            if (q + h <= N - 1) pr = q + h;
-          } else {
-            const int mm = ((N - 1) >> (lvl - 1)) << (lvl - 1);
-            if (ctz32(mm) == lvl - 1) pl = mm;
-          }
-          if (pl) z = row_dot_sub<NB>(m.Lr + (sb + (N - pl)) * NB2 + i * NB, m.y + (sb + (N - pl)) * NB, z);
-          if (pr) z = row_dot_sub<NB>(m.Ll + (sb + (N - pr)) * NB2 + i * NB, m.y + (sb + (N - pr)) * NB, z);
+                                         int CS, float *sbuf) {
+  if constexpr (SubCfg<NB>::PAIR) {
+    fwd_tail_pair<NB>(m, rhs, s, crank, CS, sbuf);
+  } else {
+    constexpr int TS = MCfg<NB>::TS, NB2 = NB * NB;
+    const Team<TS> tm;
+    const int TEAMS = blockDim.x / TS;
+    float (*sY)[NB] = reinterpret_cast<float(*)[NB]>(sbuf);
+    const int N = m.N, Lc = m.Lc;
+    const size_t sb = (size_t)s * N;
+    const int i = tm.lane;
+    const bool xmode = coupled(m);
+    for (int lvl = 0; lvl <= Lc; ++lvl) {
+      const bool lastlvl = lvl == Lc;
+      const int ntask = lastlvl ? 1 : (lvl == 0 ? N / 2 : ((N - 1) >> lvl) + 1);
+      for (int t = crank * TEAMS + tm.id; t < ntask; t += CS * TEAMS) {
+        int q;
+        if (lastlvl) q = N;
+        else if (lvl == 0) q = 2 * t + 1;
+        else {
+          const int cnt = (N - 1) >> lvl;
+          q = t < cnt ? (t + 1) << lvl : N;
         }
-      }
-      if (!elim) {
-        if (i < NB) m.zt[zoff + i] = z;
-        continue;
-      }
-      if constexpr (!kEarly) {
-        load_row<NB>(Lrow, m.Ld + (sb + (N - q)) * NB2 + (i < NB ? i : 0) * NB);
-        inv = i < NB ? m.invd[zoff + i] : 0.0f;
-      }
-      if (TS <= 32) {
+        const bool elim = lastlvl || (q < N && ctz32(q) == lvl);
+        const size_t zoff = (sb + (N - q)) * NB;
+        // row i of L_qq and 1/L_ii: for NB <= 16 loaded first, so that they
+        // share the gather's memory round trip (in bounds for every q); for
+        // larger blocks after it (loaded first they slowed the nb = 48 solve)
+        constexpr bool kEarly = NB <= 16;
+        float Lrow[NB];
+        float inv = 0.0f;
+        if constexpr (kEarly) {
+          load_row<NB>(Lrow, m.Ld + (sb + (N - q)) * NB2 + (i < NB ? i : 0) * NB);
+          inv = i < NB ? m.invd[zoff + i] : 0.0f;
+        }
+        float z = 0.0f;
+        if (i < NB) {
+          z = (lvl <= 1) ? __double2float_rn(rhs[zoff + i]) : __ldcg(m.zt + zoff + i);
+          if (lvl >= 1) {
+            const int h = 1 << (lvl - 1);
+            int pl = 0, pr = 0;
+            if (q < N) {
+              pl = q - h;
+              if (q + h <= N - 1) pr = q + h;
+            } else {
+              const int mm = ((N - 1) >> (lvl - 1)) << (lvl - 1);
+              if (ctz32(mm) == lvl - 1) pl = mm;
+            }
+            if (pl) z = row_dot_sub<NB>(m.Lr + (sb + (N - pl)) * NB2 + i * NB, m.y + (sb + (N - pl)) * NB, z);
+            if (pr) z = row_dot_sub<NB>(m.Ll + (sb + (N - pr)) * NB2 + i * NB, m.y + (sb + (N - pr)) * NB, z);
+          }
+        }
+        if (!elim) {
+          if (i < NB) m.zt[zoff + i] = z;
+          continue;
+        }
+        if constexpr (!kEarly) {
+          load_row<NB>(Lrow, m.Ld + (sb + (N - q)) * NB2 + (i < NB ? i : 0) * NB);
+          inv = i < NB ? m.invd[zoff + i] : 0.0f;
+        }
         const int base = (threadIdx.x & 31) & ~(TS - 1);
 #pragma unroll
         for (int j = 0; j < NB; ++j) {
@@ -301,35 +492,25 @@ __device__ __forceinline__ void fwd_tail(const MixedState &m, const double *__re
         }
         if (i < NB) sY[tm.id][i] = z;
         tm.sync();
-      } else {
-#pragma unroll
-        for (int j = 0; j < NB; ++j) {
-          if (i == j) {
-            z *= inv;
-            sY[tm.id][j] = z;
-          }
+        if (i < NB) m.y[zoff + i] = z;
+        if (lastlvl && !xmode) {
           tm.sync();
-          if (i > j && i < NB) z = fmaf(-Lrow[j], sY[tm.id][j], z);
-        }
-      }
-      if (i < NB) m.y[zoff + i] = z;
-      if (lastlvl && !xmode) {
-        tm.sync();
-        const int nr = m.nr;
-        const double *Fs = m.F + (size_t)s * nr * NB;
-        for (int c = i; c < nr; c += TS) {
-          double acc = 0.0;
+          const int nr = m.nr;
+          const double *Fs = m.F + (size_t)s * nr * NB;
+          for (int c = i; c < nr; c += TS) {
+            double acc = 0.0;
 #pragma unroll
-          for (int k = 0; k < NB; ++k) acc = fma(Fs[c * NB + k], f2d_exact(sY[tm.id][k]), acc);
-          m.tb[(size_t)s * nr + c] = acc;
+            for (int k = 0; k < NB; ++k) acc = fma(Fs[c * NB + k], f2d_exact(sY[tm.id][k]), acc);
+            m.tb[(size_t)s * nr + c] = acc;
+          }
         }
+        tm.sync();
       }
-      tm.sync();
+      if (CS > 1)
+        cluster_sync();
+      else
+        __syncthreads();
     }
-    if (CS > 1)
-      cluster_sync();
-    else
-      __syncthreads();
   }
 }
 
@@ -388,19 +569,45 @@ __device__ __forceinline__ bool last_cta(unsigned *ticket, unsigned n) {
   return last != 0;
 }
 
-// Backward substitution in FP32 fused with x += d (FP64); the correction of
-// each position overwrites its forward vector y.
+// The correction of a row, z, into y, x (xo before) and the planes of x.
+__device__ __forceinline__ void bwd_store(const MixedState &m, double *x, int iter, size_t row, float z, double xo,
+                                          bool xmode, const float *sdh, const float *sdl) {
+  m.y[row] = z;
+  double dz;
+  if (xmode) {
+    // d_i = z - X_i d_0 on this row, the product summed by Dot2
+    const float *xr = m.Xc + row * m.ldc;
+    float h = 0.0f, l = 0.0f;
+    for (int c = 0; c < m.nr; ++c) ff::dot2_step_split(h, l, sdh[c], sdl[c], __ldcg(xr + c));
+    float dh, e;
+    ff::two_sum(z, -h, dh, e);
+    dz = ff::to_double(dh, __fsub_rn(e, l));
+  } else {
+    dz = f2d_exact(z);
+  }
+  const double xv = iter == 0 ? dz : xo + dz;
+  x[row] = xv;
+  if (m.ffres) {
+    float h, l;
+    ff::split_d(xv, h, l);
+    m.xh[row] = h;
+    m.xl[row] = l;
+    if (ff::out_of_range(xv)) m.status->ffbad = 1;
+  }
+}
+
 template <int NB>
-__device__ __forceinline__ void bwd_tail(const MixedState &m, double *x, int iter, int s, int crank, int CS,
-                                         float (*sX)[NB]) {
-  constexpr int TS = MCfg<NB>::TS, TEAMS = MCfg<NB>::TEAMS, NB2 = NB * NB;
-  const Team<TS> tm;
+__device__ __forceinline__ void bwd_tail_pair(const MixedState &m, double *x, int iter, int s, int crank, int CS,
+                                              float *sbuf) {
+  constexpr int NB2 = NB * NB;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, teams = blockDim.x >> 5;
+  const bool two = lane + 32 < NB;
+  const int i0 = lane, i1 = two ? lane + 32 : lane;
   const int N = m.N, Lc = m.Lc, nr = m.nr;
   const size_t sb = (size_t)s * N;
-  const int i = tm.lane;
+  float *buf = sbuf + warp * SubCfg<NB>::BLK;
   const bool xmode = coupled(m);
-  // d_0 as hi + lo floats for the tails' X_i d_0 (refined coupling columns)
-  __shared__ float sdh[64], sdl[64];
+  __shared__ float sdh[64], sdl[64];   // d_0 as hi + lo floats (refined coupling columns)
   if (xmode) {
     for (int c = threadIdx.x; c < nr; c += blockDim.x) ff::split_d(__ldcg(m.d0 + c), sdh[c], sdl[c]);
     __syncthreads();
@@ -408,92 +615,144 @@ __device__ __forceinline__ void bwd_tail(const MixedState &m, double *x, int ite
   for (int lvl = Lc; lvl >= 0; --lvl) {
     const bool first = lvl == Lc;
     const int ntask = first ? 1 : (((N - 1) >> lvl) + 1) / 2;
-    for (int t = crank * TEAMS + tm.id; t < ntask; t += CS * TEAMS) {
+    for (int t = crank * teams + warp; t < ntask; t += CS * teams) {
       const int q = first ? N : (2 * t + 1) << lvl;
-      const size_t zoff = (sb + (N - q)) * NB;
-      // column i of L_qq and 1/L_ii: loaded with the gather's operands for
-      // NB <= 16, after the gather for larger blocks
-      constexpr bool kEarly = NB <= 16;
-      float Lcol[NB];
-      float inv = 0.0f;
-      if constexpr (kEarly) {
-        const float *Ld = m.Ld + (sb + (N - q)) * NB2 + (i < NB ? i : 0);
-#pragma unroll
-        for (int k = 0; k < NB; ++k) Lcol[k] = Ld[k * NB];
-        inv = i < NB ? m.invd[zoff + i] : 0.0f;
+      const size_t pos = sb + (N - q), zoff = pos * NB;
+      pair_stage<NB>(buf, m.Ld + pos * NB2);
+      const float inv0 = m.invd[zoff + i0], inv1 = m.invd[zoff + i1];
+      const double x0 = iter == 0 ? 0.0 : x[zoff + i0], x1 = iter == 0 ? 0.0 : x[zoff + i1];
+      float z0 = m.y[zoff + i0], z1 = m.y[zoff + i1];
+      if (!first) {
+        const int h = 1 << lvl;
+        const int a = q - h, b = (q + h <= N - 1) ? q + h : N;
+        pair_col_dot<NB>(m.Lr + pos * NB2 + i0, two, m.y + (sb + (N - b)) * NB, z0, z1);
+        if (q > h) pair_col_dot<NB>(m.Ll + pos * NB2 + i0, two, m.y + (sb + (N - a)) * NB, z0, z1);
+      } else if (!xmode) {
+        const double *Fs = m.F + (size_t)s * nr * NB;
+        double d0 = f2d_exact(z0), d1 = f2d_exact(z1);
+        for (int c = 0; c < nr; ++c) {
+          const double v = __ldcg(m.d0 + c);
+          d0 = fma(-Fs[c * NB + i0], v, d0);
+          d1 = fma(-Fs[c * NB + i1], v, d1);
+        }
+        z0 = __double2float_rn(d0);
+        z1 = __double2float_rn(d1);
       }
-      float z = 0.0f;
-      if (i < NB) {
-        if (first && xmode) {
-          z = m.y[zoff + i];
-        } else if (first) {
-          double zd = f2d_exact(m.y[zoff + i]);
-          const double *Fs = m.F + (size_t)s * nr * NB;
-          for (int c = 0; c < nr; ++c) zd = fma(-Fs[c * NB + i], __ldcg(m.d0 + c), zd);
-          z = __double2float_rn(zd);
+      rows::cp_async_wait();
+      __syncwarp();
+#pragma unroll
+      for (int j = NB - 1; j >= 0; --j) {
+        float xj;
+        if (j >= 32) {
+          if (lane == j - 32) z1 *= inv1;
+          xj = __shfl_sync(0xffffffffu, z1, j - 32);
+          if (lane < j - 32) z1 = fmaf(-buf[SubCfg<NB>::row(j) + i1], xj, z1);
+          z0 = fmaf(-buf[SubCfg<NB>::row(j) + i0], xj, z0);
         } else {
-          z = m.y[zoff + i];
-          const int h = 1 << lvl;
-          const int a = q - h, b = (q + h <= N - 1) ? q + h : N;
-          z = col_dot_sub<NB>(m.Lr + (sb + (N - q)) * NB2 + i, m.y + (sb + (N - b)) * NB, z);
-          if (q > h) z = col_dot_sub<NB>(m.Ll + (sb + (N - q)) * NB2 + i, m.y + (sb + (N - a)) * NB, z);
+          if (i0 == j) z0 *= inv0;
+          xj = __shfl_sync(0xffffffffu, z0, j);
+          if (i0 < j) z0 = fmaf(-buf[SubCfg<NB>::row(j) + i0], xj, z0);
         }
       }
-      if constexpr (!kEarly) {
-        const float *Ld = m.Ld + (sb + (N - q)) * NB2 + (i < NB ? i : 0);
-#pragma unroll
-        for (int k = 0; k < NB; ++k) Lcol[k] = Ld[k * NB];
-        inv = i < NB ? m.invd[zoff + i] : 0.0f;
-      }
-      if (TS <= 32) {
-        const int base = (threadIdx.x & 31) & ~(TS - 1);
-#pragma unroll
-        for (int j = NB - 1; j >= 0; --j) {
-          if (i == j) z *= inv;
-          const float xj = __shfl_sync(tm.mask, z, base + j);
-          if (i < j) z = fmaf(-Lcol[j], xj, z);
-        }
-      } else {
-#pragma unroll
-        for (int j = NB - 1; j >= 0; --j) {
-          if (i == j) {
-            z *= inv;
-            sX[tm.id][j] = z;
-          }
-          tm.sync();
-          if (i < j) z = fmaf(-Lcol[j], sX[tm.id][j], z);
-        }
-      }
-      if (i < NB) {
-        m.y[zoff + i] = z;
-        double dz;
-        if (xmode) {
-          // d_i = z - X_i d_0 on this row, the product summed by Dot2
-          const float *xr = m.Xc + (zoff + i) * m.ldc;
-          float h = 0.0f, l = 0.0f;
-          for (int c = 0; c < nr; ++c) ff::dot2_step_split(h, l, sdh[c], sdl[c], __ldcg(xr + c));
-          float dh, e;
-          ff::two_sum(z, -h, dh, e);
-          dz = ff::to_double(dh, __fsub_rn(e, l));
-        } else {
-          dz = f2d_exact(z);
-        }
-        const double xv = iter == 0 ? dz : x[zoff + i] + dz;
-        x[zoff + i] = xv;
-        if (m.ffres) {
-          float h, l;
-          ff::split_d(xv, h, l);
-          m.xh[zoff + i] = h;
-          m.xl[zoff + i] = l;
-          if (ff::out_of_range(xv)) m.status->ffbad = 1;
-        }
-      }
-      tm.sync();
+      bwd_store(m, x, iter, zoff + i0, z0, x0, xmode, sdh, sdl);
+      if (two) bwd_store(m, x, iter, zoff + i1, z1, x1, xmode, sdh, sdl);
     }
     if (CS > 1)
       cluster_sync();
     else
       __syncthreads();
+  }
+}
+
+// Backward substitution in FP32 fused with x += d (FP64); the correction of
+// each position overwrites its forward vector y.
+template <int NB, bool PAIR = SubCfg<NB>::PAIR>
+__device__ __forceinline__ void bwd_tail(const MixedState &m, double *x, int iter, int s, int crank, int CS,
+                                         float *sbuf) {
+  if constexpr (PAIR) {
+    bwd_tail_pair<NB>(m, x, iter, s, crank, CS, sbuf);
+  } else {
+    constexpr int TS = MCfg<NB>::TS, NB2 = NB * NB;
+    const Team<TS> tm;
+    const int TEAMS = blockDim.x / TS;
+    const int N = m.N, Lc = m.Lc, nr = m.nr;
+    const size_t sb = (size_t)s * N;
+    const int i = tm.lane;
+    const bool xmode = coupled(m);
+    // d_0 as hi + lo floats for the tails' X_i d_0 (refined coupling columns)
+    __shared__ float sdh[64], sdl[64];
+    if (xmode) {
+      for (int c = threadIdx.x; c < nr; c += blockDim.x) ff::split_d(__ldcg(m.d0 + c), sdh[c], sdl[c]);
+      __syncthreads();
+    }
+    for (int lvl = Lc; lvl >= 0; --lvl) {
+      const bool first = lvl == Lc;
+      const int ntask = first ? 1 : (((N - 1) >> lvl) + 1) / 2;
+      for (int t = crank * TEAMS + tm.id; t < ntask; t += CS * TEAMS) {
+        const int q = first ? N : (2 * t + 1) << lvl;
+        const size_t zoff = (sb + (N - q)) * NB;
+        // column i of L_qq and 1/L_ii: loaded with the gather's operands for
+        // NB <= 16, after the gather for larger blocks
+        constexpr bool kEarly = NB <= 16;
+        float Lcol[NB];
+        float inv = 0.0f;
+        if constexpr (kEarly) {
+          const float *Ld = m.Ld + (sb + (N - q)) * NB2 + (i < NB ? i : 0);
+#pragma unroll
+          for (int k = 0; k < NB; ++k) Lcol[k] = Ld[k * NB];
+          inv = i < NB ? m.invd[zoff + i] : 0.0f;
+        }
+        float z = 0.0f;
+        if (i < NB) {
+          if (first && xmode) {
+            z = m.y[zoff + i];
+          } else if (first) {
+            double zd = f2d_exact(m.y[zoff + i]);
+            const double *Fs = m.F + (size_t)s * nr * NB;
+            for (int c = 0; c < nr; ++c) zd = fma(-Fs[c * NB + i], __ldcg(m.d0 + c), zd);
+            z = __double2float_rn(zd);
+          } else {
+            z = m.y[zoff + i];
+            const int h = 1 << lvl;
+            const int a = q - h, b = (q + h <= N - 1) ? q + h : N;
+            z = col_dot_sub<NB>(m.Lr + (sb + (N - q)) * NB2 + i, m.y + (sb + (N - b)) * NB, z);
+            if (q > h) z = col_dot_sub<NB>(m.Ll + (sb + (N - q)) * NB2 + i, m.y + (sb + (N - a)) * NB, z);
+          }
+        }
+        if constexpr (!kEarly) {
+          const float *Ld = m.Ld + (sb + (N - q)) * NB2 + (i < NB ? i : 0);
+#pragma unroll
+          for (int k = 0; k < NB; ++k) Lcol[k] = Ld[k * NB];
+          inv = i < NB ? m.invd[zoff + i] : 0.0f;
+        }
+        if constexpr (TS <= 32) {
+          const int base = (threadIdx.x & 31) & ~(TS - 1);
+#pragma unroll
+          for (int j = NB - 1; j >= 0; --j) {
+            if (i == j) z *= inv;
+            const float xj = __shfl_sync(tm.mask, z, base + j);
+            if (i < j) z = fmaf(-Lcol[j], xj, z);
+          }
+        } else {
+          float *sX = sbuf + tm.id * NB;
+#pragma unroll
+          for (int j = NB - 1; j >= 0; --j) {
+            if (i == j) {
+              z *= inv;
+              sX[j] = z;
+            }
+            tm.sync();
+            if (i < j) z = fmaf(-Lcol[j], sX[j], z);
+          }
+        }
+        if (i < NB) bwd_store(m, x, iter, zoff + i, z, iter == 0 ? 0.0 : x[zoff + i], xmode, sdh, sdl);
+        tm.sync();
+      }
+      if (CS > 1)
+        cluster_sync();
+      else
+        __syncthreads();
+    }
   }
 }
 
