@@ -65,8 +65,9 @@ __global__ void __launch_bounds__(256, 3) k_batch_bwd(const BInst *inst, const B
   }
 }
 
-__global__ void __launch_bounds__(256) k_batch_res(const BInst *inst, const BTail *tails, const double *const *rp,
-                                                   double *const *xp, int iter, int max_iter, double tol) {
+__global__ void __launch_bounds__(256, 3) k_batch_res(const BInst *inst, const BTail *tails, const double *const *rp,
+                                                      double *const *xp, int iter, int max_iter, double tol) {
+  __shared__ double sbuf[8 * ResCfg<48>::WARP];
   const BTail t = tails[blockIdx.x];
   const BInst &I = inst[t.inst];
   pdl_wait();
@@ -76,7 +77,7 @@ __global__ void __launch_bounds__(256) k_batch_res(const BInst *inst, const BTai
   switch (I.nb) {
 #define X(n)                                     \
   case n:                                        \
-    residual_tail<n>(I.m, r, x, t.s);            \
+    residual_tail<n>(I.m, r, x, t.s, sbuf);      \
     break;
     BM_BATCH_NB_LIST(X)
 #undef X

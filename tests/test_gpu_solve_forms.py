@@ -47,10 +47,11 @@ def test_few_tails_form_gives_the_cluster_kernels_bits(S, N, nb):
 
 
 # few tails in one CTA each; blocks of 48 with a warp per position, over
-# clusters and one CTA per tail
+# clusters and one CTA per tail; the batch's staged FP64 residual where the
+# tail's rows are not a multiple of 32
 @pytest.mark.parametrize("S,N,nb", [(304, 1, 4), (304, 2, 4), (304, 8, 6), (304, 33, 12), (304, 40, 24), (152, 13, 48),
-                                    (160, 1, 48), (160, 9, 48), (3, 64, 48), (2, 45, 48), (3, 3, 24)])
-def test_substitutions_give_the_batched_forms_bits(S, N, nb, tmp_path, monkeypatch):
+                                    (160, 1, 48), (160, 9, 48), (3, 64, 48), (2, 45, 48), (3, 3, 24), (5, 7, 24)])
+def test_substitutions_and_residuals_give_the_batched_forms_bits(S, N, nb, tmp_path, monkeypatch):
     import paper_2609_29977_gb300 as bm
     monkeypatch.setenv("BM_AUTOTUNE_CACHE", str(tmp_path / "tune.json"))
     d = _system(S, N, nb)
