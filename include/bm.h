@@ -413,10 +413,11 @@ void bm_destroy(bm_handle h);
  * nrhs solves of Alg. 2 against the resident factor) on its own stream slot
  * so that the work of requests admitted at different times overlaps on the
  * GPU, and reports per-request latency. Not in the paper: the paper solves
- * one system at a time. A request is computed exactly as bm_factor /
- * bm_solve compute it alone (same kernels, same launch shapes, which depend
- * only on the request's shape), so its result does not depend on what else
- * is in flight.
+ * one system at a time. A request is computed as bm_factor / bm_solve
+ * compute it alone (same kernels and launch shapes, which depend only on the
+ * request's shape; of a solve's refinement iterations the first five are
+ * launched at once and the rest when a right-hand side needs them, with the
+ * same bits), so its result does not depend on what else is in flight.
  *
  * Admission is first-in first-out: the request at the head of the queue is
  * admitted as soon as a slot is free and a contiguous range of the server's

@@ -384,7 +384,7 @@ __device__ __forceinline__ void x1_task_w(const TailView<float> &v, void *sbuf, 
 
 // Grid-wide level: one team per CTA (seven CTAs per SM).
 template <int NB>
-__global__ void __launch_bounds__(96, 7) k_level_w(TailView<float> v, int lvl) {
+__global__ void __launch_bounds__(96, 7) k_level_rows_w(TailView<float> v, int lvl) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int N = v.N, S = v.S, lane = threadIdx.x;
   const int E = level_elims(N, lvl);
@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(96, 7) k_level_w(TailView<float> v, int lvl) {
 
 // Top levels lvl0..Lc-1 and x_1 of one tail per CTA.
 template <int NB>
-__global__ void __launch_bounds__(4 * 96) k_top_w(TailView<float> v, int lvl0) {
+__global__ void __launch_bounds__(4 * 96) k_top_rows_w(TailView<float> v, int lvl0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int TS = WCfg<NB>::TS;
   const int team = threadIdx.x / TS, lane = threadIdx.x - team * TS, teams = blockDim.x / TS;
@@ -431,9 +431,9 @@ __global__ void __launch_bounds__(4 * 96) k_top_w(TailView<float> v, int lvl0) {
 
 template <int NB>
 cudaError_t prepare_w() {
-  cudaError_t e = cudaFuncSetAttribute(k_level_w<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+  cudaError_t e = cudaFuncSetAttribute(k_level_rows_w<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_top_w<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  return cudaFuncSetAttribute(k_top_rows_w<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }
 
 template <int NB>
@@ -443,7 +443,7 @@ void launch_tail_w(const TailView<float> &v, cudaStream_t st) {
   for (int l = 0; l < Tl; ++l) {
     const int E = level_elims(v.N, l);
     const int G = l == 0 ? 0 : ((v.N - 1) >> (l + 1)) + 1;
-    launch_pdl(k_level_w<NB>, (unsigned)((long)v.S * (E + G)), 96, per, st, v, l);
+    launch_pdl(k_level_rows_w<NB>, (unsigned)((long)v.S * (E + G)), 96, per, st, v, l);
   }
   // four teams per tail while every SM has a tail to itself, fewer with more
   // tails than that: the shared memory then holds more tails, and one
@@ -452,7 +452,7 @@ void launch_tail_w(const TailView<float> &v, cudaStream_t st) {
   size_t smem = teams * per;
   const size_t x1b = x1_w_bytes<NB>(v.nr);
   if (x1b > smem) smem = x1b;
-  launch_pdl(k_top_w<NB>, (unsigned)v.S, teams * 96, smem, st, v, Tl);
+  launch_pdl(k_top_rows_w<NB>, (unsigned)v.S, teams * 96, smem, st, v, Tl);
 }
 
 }  // namespace rows
