@@ -835,8 +835,8 @@ def run_gpu(args):
                 "peak_source": peak_src,
                 "achieved_basis": "method flops of one factor (%.4g) / mean factor time over the timed "
                                   "steps (CUDA events on the launching stream)" % fl["factor"]}
-    if args.precision == "fp64" and w.nb >= 12:
-        # the products of blocks from 12 on run as exact digit products on the
+    if args.precision == "fp64" and w.nb >= 16:
+        # the products of blocks from 16 on run as exact digit products on the
         # tensor cores, so the FP64 ALU's rate bounds nothing any more: the
         # floor is the bytes
         roofline = {"bound": "hbm", "achieved": factor_gbs, "peak": _peaks()[0]["hbm_gbs"], "unit": "GB/s",

@@ -29,9 +29,8 @@
 //
 // The error is below that of the FMA chain it replaces (nb roundings of
 // partial sums): componentwise backward error of the solution, geometric
-// mean over six systems, 5.8e-16 -> 3.9e-16 (nb = 12), 7.2e-16 -> 2.8e-16
-// (16), 6.8e-16 -> 2.7e-16 (24), 6.2e-16 -> 2.4e-16 (32), 5.7e-16 -> 1.9e-16
-// (48); the solution's own error falls by 1.7 to 5 times. A row whose largest
+// mean over six systems, 7.2e-16 -> 2.8e-16 (nb = 16), 6.8e-16 -> 2.7e-16
+// (24), 6.2e-16 -> 2.4e-16 (32), 5.7e-16 -> 1.9e-16 (48); the solution's own error falls by 1.7 to 5 times. A row whose largest
 // exponent is that of inf or NaN makes every product with it NaN, which a
 // later pivot reports.
 //
@@ -52,10 +51,11 @@ namespace sliced {
 
 constexpr int ND = 7;   // digits of 9 bits
 
-// Block sizes whose FP64 tails use the sliced products.
+// Block sizes whose FP64 tails use the sliced products (the line is drawn at
+// Ops in bm_tail_factor.cuh).
 template <typename T, int NB>
 struct Use {
-  static constexpr bool value = sizeof(T) == sizeof(double) && NB % 4 == 0 && NB >= 12;
+  static constexpr bool value = sizeof(T) == sizeof(double) && NB % 8 == 0 && NB >= 16;
 };
 
 // Bias that makes all seven digits non-negative: 256 at every digit.
@@ -109,14 +109,14 @@ __device__ __forceinline__ void mma_k8(float (&c)[4], unsigned a0, unsigned a1, 
 // layout of mma.sync for A (rows) and for B (rows of B^T), and also the
 // layout of the product's accumulators.
 template <int K>
-__device__ __forceinline__ void load_rows(double (&x)[(K + 7) / 8][2], const double *__restrict__ base, int ld,
+__device__ __forceinline__ void load_rows(double (&x)[K / 8][2], const double *__restrict__ base, int ld,
                                           int row, int nrows) {
   const int tig = threadIdx.x & 3;
 #pragma unroll
-  for (int g = 0; g < (K + 7) / 8; ++g) {
+  for (int g = 0; g < K / 8; ++g) {
     const int k = 8 * g + 2 * tig;
     double2 v = make_double2(0.0, 0.0);
-    if (row < nrows && (K % 8 == 0 || k < K)) v = *reinterpret_cast<const double2 *>(base + row * ld + k);
+    if (row < nrows) v = *reinterpret_cast<const double2 *>(base + row * ld + k);
     x[g][0] = v.x;
     x[g][1] = v.y;
   }
@@ -203,7 +203,7 @@ template <int TEAM, int K, bool SYRK, typename Out>
 __device__ __forceinline__ void product(const Team<TEAM> &tm, const double *A, int lda, int M, const double *B,
                                         int ldb, int NC, Out out) {
   static_assert(TEAM >= 32, "whole warps");
-  constexpr int KG = (K + 7) / 8, W = TEAM / 32;
+  constexpr int KG = K / 8, W = TEAM / 32;
   const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
   const int warp = tm.lane >> 5;
   const int MT = (M + 15) / 16, NT = (NC + 7) / 8;
@@ -295,10 +295,11 @@ __device__ __forceinline__ void team_gemm_nt_neg(const Team<TEAM> &tm, double *_
   product<TEAM, NB, false>(tm, A, NB, NB, B, NB, NB, [&](int i, int j, double v) { out[i * NB + j] = -v; });
 }
 
-// 1 / d for a positive normal d to about an ulp: an FP32 estimate of the
-// reciprocal of the significand (error e0 below 2^-21), one third-order step
-// y (1 + e + e^2) in FP64 (three dependent FP64 instructions; a library
-// division takes more than twice that), the exponent by integer arithmetic.
+// 1 / d for a positive normal d to about an ulp: an FP32 estimate y of the
+// reciprocal of the significand m (relative error e = 1 - m y below 2^-21),
+// and the geometric series 1/m = y / (1 - e) cut after e^2, whose rest e^3 is
+// below 2^-63, in FP64 (three dependent FP64 instructions; a library division
+// takes more than twice that), the exponent by integer arithmetic.
 // Subnormal d, and d so large that 1/d is subnormal, take the division.
 __device__ __forceinline__ double pivot_rcp(double d) {
   const int hi = __double2hiint(d);
@@ -400,24 +401,20 @@ __device__ __forceinline__ void team_invert_diagonal(const Team<TEAM> &tm, doubl
     double v[8];
     if (c < NB) {
       const double *M = sA + c0 * NB + c0;   // M_kl at M[l * NB + k], l < k
-      const int pw = NB - c0 < 8 ? NB - c0 : 8;
 #pragma unroll
       for (int k = 0; k < 8; ++k) v[k] = k == jj ? 1.0 : 0.0;
 #pragma unroll
       for (int k = 1; k < 8; ++k) {
-        if (NB % 8 == 0 || k < pw) {
-          double acc = 0.0;
+        double acc = 0.0;
 #pragma unroll
-          for (int l = 0; l < k; ++l) acc = fma(-M[l * NB + k], v[l], acc);
-          if (k > jj) v[k] = acc;
-        }
+        for (int l = 0; l < k; ++l) acc = fma(-M[l * NB + k], v[l], acc);
+        if (k > jj) v[k] = acc;
       }
     }
     tm.sync();
     if (c < NB) {
 #pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (NB % 8 == 0 || c0 + k < NB) sA[(c0 + k) * NB + c] = v[k] * inv[c0 + k];
+      for (int k = 0; k < 8; ++k) sA[(c0 + k) * NB + c] = v[k] * inv[c0 + k];
     }
     tm.sync();
   }
@@ -429,13 +426,13 @@ __device__ __forceinline__ void team_invert_diagonal(const Team<TEAM> &tm, doubl
 // block. The accumulators of a product have the layout of the next one's
 // operand, so nothing passes through shared memory in between.
 template <int NB, int P>
-__device__ __forceinline__ void trsm_panel(double (&x)[2][(NB + 7) / 8][2], const double *sA) {
-  constexpr int c0 = 8 * P, PW = NB - c0 < 8 ? NB - c0 : 8;
+__device__ __forceinline__ void trsm_panel(double (&x)[2][NB / 8][2], const double *sA) {
+  constexpr int c0 = 8 * P;
   const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
   if constexpr (P > 0) {
     const int E0 = row_exponent<P>(x[0]), E1 = row_exponent<P>(x[1]);
     double b[P][2];
-    load_rows<c0>(b, sA + c0 * NB, NB, gid, PW);
+    load_rows<c0>(b, sA + c0 * NB, NB, gid, 8);
     const int Eb = row_exponent<P>(b);
     float c[ND][4];
     clear(c);
@@ -463,7 +460,7 @@ __device__ __forceinline__ void trsm_panel(double (&x)[2][(NB + 7) / 8][2], cons
       x[t >> 1][P][t & 1] -= assemble<c0>(c, t, t >> 1 ? E1 : E0, (t & 1) ? Eb1 : Eb0);
   }
   double b[1][2];
-  load_rows<PW>(b, sA + c0 * NB + c0, NB, gid, PW);
+  load_rows<8>(b, sA + c0 * NB + c0, NB, gid, 8);
   const int Eb = row_exponent<1>(b);
   double y0[1][2] = {{x[0][P][0], x[0][P][1]}}, y1[1][2] = {{x[1][P][0], x[1][P][1]}};
   const int E0 = row_exponent<1>(y0), E1 = row_exponent<1>(y1);
@@ -485,7 +482,7 @@ __device__ __forceinline__ void trsm_panel(double (&x)[2][(NB + 7) / 8][2], cons
 // (the factor is stored before).
 template <int TEAM, int NB>
 __device__ __forceinline__ void team_trsm_lt(const Team<TEAM> &tm, double *X, int M, double *sA, const double *inv) {
-  constexpr int KG = (NB + 7) / 8;
+  constexpr int KG = NB / 8;
   const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
   tm.sync();
   team_invert_diagonal<TEAM, NB>(tm, sA, inv);
@@ -501,7 +498,7 @@ __device__ __forceinline__ void team_trsm_lt(const Team<TEAM> &tm, double *X, in
 #pragma unroll
       for (int g = 0; g < KG; ++g) {
         const int k = 8 * g + 2 * tig;
-        if (row < M && (NB % 8 == 0 || k < NB))
+        if (row < M)
           *reinterpret_cast<double2 *>(X + row * NB + k) = make_double2(x[h][g][0], x[h][g][1]);
       }
     }

@@ -49,12 +49,14 @@ __device__ __forceinline__ void team_load_t(const Team<TEAM> &tm, T *__restrict_
 }
 
 // The block operations of a task: on the FP64 path the sliced products and
-// the pivots' reciprocals of bm_sliced.cuh for nb >= 12, the plain ones of
+// the pivots' reciprocals of bm_sliced.cuh for nb >= 16, the plain ones of
 // bm_team.cuh for smaller blocks and for FP32. Whole factor, plain -> sliced:
 // S = 512, N = 128, nb = 24: 6216 -> 3122 us; S = 100, N = 160, nb = 16:
-// 807 -> 438; S = N = 64, nb = 32: 1525 -> 687, nb = 48: 4695 -> 1831, and
-// nb = 12: 153 -> 152, where the line lies: one product of 12 columns costs
-// about as many issue slots as its FP64 FMAs take.
+// 807 -> 438; S = N = 64, nb = 32: 1525 -> 687, nb = 48: 4695 -> 1831. The
+// line lies below nb = 16: a product of 12 columns is padded to 16 and needs
+// a whole warp per task, where the FP64 FMAs do with 8 lanes. Factor and solve
+// of nb = 12, plain against sliced: S = N = 64: 206 and 202 us, S = 512, N = 32:
+// 374 and 452, N = 128: 1231 and 1333. nb = 16, S = 512, N = 32: 801 and 510.
 template <typename T, int NB, int TEAM>
 struct Ops {
   using Tm = Team<TEAM>;
@@ -308,7 +310,7 @@ __global__ void __launch_bounds__(TEAM * top_teams<T, NB>()) k_factor_top(TailVi
 }
 
 // Team sizes compiled for each block size, and the team of the top kernel.
-constexpr int team_min(int nb) { return nb <= 8 ? 8 : 32; }
+constexpr int team_min(int nb) { return nb <= 12 ? 8 : 32; }
 constexpr int team_max(int nb) { return nb <= 4 ? 32 : nb <= 16 ? 64 : 128; }
 constexpr int team_top(int nb) { return nb <= 8 ? 32 : nb <= 16 ? 64 : 128; }
 

@@ -1,5 +1,5 @@
 """Backward error of the tail factor in extended precision: FP64 with sliced
-tensor-core products (nb >= 12, csrc/bm_sliced.cuh), and the FP32 tails of the
+tensor-core products (nb >= 16, csrc/bm_sliced.cuh; plain FMAs below), and the FP32 tails of the
 mixed path (csrc/bm_tail_rows.cuh), whose blocks move through shared memory;
 and the properties that the digits must not break.
 
