@@ -19,20 +19,26 @@
 //     and FP32 accumulation in mma.sync (f16 operands) is exact. For nb = 48
 //     only the sums of s = 5, 6 can exceed 2^24, and then by rounding a unit
 //     that is 2^-61 of the largest product.
-//   * the pairs with i + j <= 6 (28 products) are kept; the rest and the
-//     truncation of q are below about 2^-60 of (largest |x_i|)(largest |y_j|).
-//   * the seven sums are put together in 64-bit integers and turned into a
-//     double by integer instructions (truncated 2^-56 below the largest
-//     product of the two rows, then rounded to nearest), so a fill block
-//     needs no FP64 instruction and an update needs one subtraction per
+//   * the pairs with i + j <= 6 (28 products) are kept. Relative to X Y, the
+//     powers of two above the largest entries of the two rows (up to twice
+//     those entries each), a term k loses at most 6 2^16 2^45 / 2^124 = 2^-60.4
+//     by the pairs left out and 2^-61 by the truncation of q, 2^-59.6 together,
+//     a sum over K terms K times that at worst (2^-55 for K = 24, 2^-54 for 48).
+//   * the seven sums are put together in 64-bit integers, at most two units
+//     short by truncation (2^-57 of X Y for K <= 24, 2^-56 above), and turned
+//     into a double by integer instructions, rounded to nearest, so a fill
+//     block needs no FP64 instruction and an update needs one subtraction per
 //     entry instead of nb (or 2 nb) FMAs.
 //
-// The error is below that of the FMA chain it replaces (nb roundings of
-// partial sums): componentwise backward error of the solution, geometric
-// mean over six systems, 7.2e-16 -> 2.8e-16 (nb = 16), 6.8e-16 -> 2.7e-16
-// (24), 6.2e-16 -> 2.4e-16 (32), 5.7e-16 -> 1.9e-16 (48); the solution's own error falls by 1.7 to 5 times. A row whose largest
-// exponent is that of inf or NaN makes every product with it NaN, which a
-// later pivot reports.
+// Where each row carries one scale the loss stays within the backward error
+// of an FMA chain, nb 2^-53 sqrt(K_ii K_jj): rows of L and of X do (|x_i| <=
+// sqrt(K_ii), whatever the units of the variables), and the operands of the
+// panels' inverses are brought to it (column_scale). Measured componentwise
+// backward error of the solution, geometric mean over six generated systems
+// whose variables have like units, FMA chain -> sliced: 7.2e-16 -> 2.8e-16
+// (nb = 16), 6.8e-16 -> 2.7e-16 (24), 6.2e-16 -> 2.4e-16 (32), 5.7e-16 ->
+// 1.9e-16 (48). A row whose largest exponent is that of inf or NaN makes
+// every product with it NaN, which a later pivot reports.
 //
 // What bounds the level kernels now (S = 128, N = 128, nb = 24, level 1, 242
 // us, 255 before the register-resident trsm): nothing alone. Four warps per
@@ -68,17 +74,16 @@ __device__ __forceinline__ unsigned long long biased_fixed(double x, int E) {
   const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
   const unsigned mh = ((unsigned)hi & 0xfffffu) | (e ? 0x100000u : 0u);
   const unsigned long long m = ((unsigned long long)mh << 32) | (unsigned)__double2loint(x);
-  int sh = E - (int)(e ? e : 1u);
-  sh = sh > 63 ? 63 : sh;
+  const unsigned sh = min((unsigned)(E - (int)(e ? e : 1u)), 63u);   // (63 too for a row of zeros, whatever its E)
   const unsigned long long q = (m << 9) >> sh;
   return hi < 0 ? kBias - q : kBias + q;
 }
 
 // The digits of two neighbouring entries as FP16 pairs, most significant
 // first (the operand registers of mma.sync m16n8k8/k16 hold two
-// neighbouring k of one row).
-__device__ __forceinline__ void digits(double x0, double x1, int E, unsigned (&d)[ND]) {
-  const unsigned long long a = biased_fixed(x0, E), b = biased_fixed(x1, E);
+// neighbouring k of one row), relative to the exponents E0 and E1.
+__device__ __forceinline__ void digits(double x0, double x1, int E0, int E1, unsigned (&d)[ND]) {
+  const unsigned long long a = biased_fixed(x0, E0), b = biased_fixed(x1, E1);
 #pragma unroll
   for (int i = 0; i < ND; ++i) {
     const int sh = 9 * (ND - 1 - i);
@@ -90,6 +95,8 @@ __device__ __forceinline__ void digits(double x0, double x1, int E, unsigned (&d
     d[i] = r;
   }
 }
+
+__device__ __forceinline__ void digits(double x0, double x1, int E, unsigned (&d)[ND]) { digits(x0, x1, E, E, d); }
 
 __device__ __forceinline__ void mma_k16(float (&c)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3,
                                         unsigned b0, unsigned b1) {
@@ -163,8 +170,8 @@ __device__ __forceinline__ void clear(float (&c)[ND][4]) {
 }
 
 // The double nearest to (sum_s c_s 2^(9(12-s))) 2^-124 2^(Ea-1022) 2^(Eb-1022)
-// after a truncation (of the sums of s = 5 and 6) at 2^-57 or less of the
-// largest possible product of the two rows. |c_s| as bounded above: the sum
+// after a truncation (of the sums of s = 5 and 6) by less than two units of V:
+// 2^-57 (K <= 24) or 2^-56 of the two rows' powers of two. |c_s| as bounded above: the sum
 // is below 2^(124 + log2 K), so the unit 2^66 (K <= 24) or 2^67 keeps the
 // 64-bit integer in range.
 template <int K>
@@ -389,10 +396,53 @@ __device__ __forceinline__ int team_chol(const Team<TEAM> &tm, double *sA, doubl
   return fail;
 }
 
-// G_p = (L_pp)^-1 for the 8 x 8 diagonal blocks of L, in place of those
-// blocks (zeros above the diagonal): L_pp^-1 = diag(1/L_jj) M_pp^-1 with the
-// unit factor M, whose inverse does not see the spread of the pivots. One
-// lane per column substitutes with M_pp (28 FMAs, all panels at once).
+// Column l of a panel in a scale-free form. The variables of a stage may have
+// different units: with K = S K' S (S diagonal) column l of a coupling block
+// carries s_l and column l of L_pp^-1 carries 1/s_l, while a digit product is
+// exact relative to the largest entries of its two rows only. Both rows are
+// brought to one scale each by the power of two 2^o_l next to L_ll, from the
+// exponent of 1/L_ll: y_l 2^-o_l (an offset of the exponents below) and
+// (L_pp^-1)_kl 2^o_l, both exact. Without it the backward error of the solve
+// grew with the spread of the units within a panel (emulated, 1e-16 at 2^0,
+// 1e-12 at 2^20, 2e-9 at 2^30). It costs 1.4% of factor and solve at S = 512,
+// N = 128, nb = 24 (3790 -> 3843 us), 0.9% at S = 100, N = 160, nb = 16 (603 -> 608).
+__device__ __forceinline__ int column_scale(double inv) { return 1023 - (__double2hiint(inv) >> 20); }   // (inv > 0)
+
+// Largest biased exponents E0, E1 of a panel's rows y0 (rows 0-7) and y1 (8-15), whose
+// entries in the lane's two columns count as x 2^-o0 and x 2^-o1; kBadRow as
+// in row_exponent.
+__device__ __forceinline__ void row_exponents_scaled(const double (&y0)[2], const double (&y1)[2], int o0, int o1,
+                                                     int &E0, int &E1) {
+  const double x[4] = {y0[0], y0[1], y1[0], y1[1]};
+  int c[4];
+  unsigned mx = 0;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const unsigned u = ((unsigned)__double2hiint(x[t]) & 0x7fffffffu) - 0x100000u;   // zero and subnormal wrap around
+    mx = max(mx, u);
+    c[t] = (int)(u >> 20) + 1 - (t & 1 ? o1 : o0);
+  }
+  if (mx >= 0x7fe00000u) {   // an entry that is not a normal number
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int h = __double2hiint(x[t]) & 0x7fffffff;
+      if (h >= 0x7ff00000) c[t] = kBadRow;
+      if (h < 0x100000) c[t] = (h | __double2loint(x[t])) ? 1 - (t & 1 ? o1 : o0) : -4096;
+    }
+  }
+  E0 = max(c[0], c[1]);
+  E1 = max(c[2], c[3]);
+#pragma unroll
+  for (int m = 1; m <= 2; m <<= 1) {
+    E0 = max(E0, __shfl_xor_sync(0xffffffffu, E0, m));
+    E1 = max(E1, __shfl_xor_sync(0xffffffffu, E1, m));
+  }
+}
+
+// G_p = (L_pp)^-1 diag(p_l) for the 8 x 8 diagonal blocks of L, in place of
+// those blocks (zeros above the diagonal): L_pp^-1 = diag(1/L_jj) M_pp^-1 with
+// the unit factor M. One lane per column substitutes with M_pp (28 FMAs, all
+// panels at once), from p_l instead of 1 (column_scale).
 template <int TEAM, int NB>
 __device__ __forceinline__ void team_invert_diagonal(const Team<TEAM> &tm, double *sA, const double *inv) {
 #pragma unroll
@@ -401,8 +451,9 @@ __device__ __forceinline__ void team_invert_diagonal(const Team<TEAM> &tm, doubl
     double v[8];
     if (c < NB) {
       const double *M = sA + c0 * NB + c0;   // M_kl at M[l * NB + k], l < k
+      const double p = __hiloint2double((1023 + column_scale(inv[c])) << 20, 0);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) v[k] = k == jj ? 1.0 : 0.0;
+      for (int k = 0; k < 8; ++k) v[k] = k == jj ? p : 0.0;
 #pragma unroll
       for (int k = 1; k < 8; ++k) {
         double acc = 0.0;
@@ -423,10 +474,11 @@ __device__ __forceinline__ void team_invert_diagonal(const Team<TEAM> &tm, doubl
 // One panel of team_trsm_lt for 16 rows held in registers (x[h][g]: rows 0-7
 // and 8-15 of the tile): the columns before the panel act on it through the
 // lower triangle of L, then it is multiplied by the inverse of its diagonal
-// block. The accumulators of a product have the layout of the next one's
-// operand, so nothing passes through shared memory in between.
+// block, both scaled per column (column_scale). The accumulators of a product
+// have the layout of the next one's operand, so nothing passes through shared
+// memory in between.
 template <int NB, int P>
-__device__ __forceinline__ void trsm_panel(double (&x)[2][NB / 8][2], const double *sA) {
+__device__ __forceinline__ void trsm_panel(double (&x)[2][NB / 8][2], const double *sA, const double *inv) {
   constexpr int c0 = 8 * P;
   const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
   if constexpr (P > 0) {
@@ -462,11 +514,12 @@ __device__ __forceinline__ void trsm_panel(double (&x)[2][NB / 8][2], const doub
   double b[1][2];
   load_rows<8>(b, sA + c0 * NB + c0, NB, gid, 8);
   const int Eb = row_exponent<1>(b);
-  double y0[1][2] = {{x[0][P][0], x[0][P][1]}}, y1[1][2] = {{x[1][P][0], x[1][P][1]}};
-  const int E0 = row_exponent<1>(y0), E1 = row_exponent<1>(y1);
+  const int o0 = column_scale(inv[c0 + 2 * tig]), o1 = column_scale(inv[c0 + 2 * tig + 1]);
+  int E0, E1;
+  row_exponents_scaled(x[0][P], x[1][P], o0, o1, E0, E1);
   unsigned a0[ND], a1[ND], bd[ND];
-  digits(y0[0][0], y0[0][1], E0, a0);
-  digits(y1[0][0], y1[0][1], E1, a1);
+  digits(x[0][P][0], x[0][P][1], E0 + o0, E0 + o1, a0);
+  digits(x[1][P][0], x[1][P][1], E1 + o0, E1 + o1, a1);
   digits(b[0][0], b[0][1], Eb, bd);
   float c[ND][4];
   clear(c);
@@ -474,7 +527,7 @@ __device__ __forceinline__ void trsm_panel(double (&x)[2][NB / 8][2], const doub
   const int Eb0 = __shfl_sync(0xffffffffu, Eb, 8 * tig), Eb1 = __shfl_sync(0xffffffffu, Eb, 8 * tig + 4);
 #pragma unroll
   for (int t = 0; t < 4; ++t) x[t >> 1][P][t & 1] = assemble<8>(c, t, t >> 1 ? E1 : E0, (t & 1) ? Eb1 : Eb0);
-  if constexpr (c0 + 8 < NB) trsm_panel<NB, P + 1>(x, sA);
+  if constexpr (c0 + 8 < NB) trsm_panel<NB, P + 1>(x, sA, inv);
 }
 
 // X (M x NB) := X L^{-T}, all of it sliced products, 16 rows per warp at a
@@ -491,7 +544,7 @@ __device__ __forceinline__ void team_trsm_lt(const Team<TEAM> &tm, double *X, in
     double x[2][KG][2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) load_rows<NB>(x[h], X, NB, mt * 16 + h * 8 + gid, M);
-    trsm_panel<NB, 0>(x, sA);
+    trsm_panel<NB, 0>(x, sA, inv);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int row = mt * 16 + h * 8 + gid;

@@ -136,3 +136,64 @@ def test_non_finite_coupling_is_reported(nb, bad):
     d["E"][1, 3, nb - 1, 2] = bad
     _, _, info = _run(d)
     assert info["name"] == "BM_ERR_NOT_SPD" and info["fail_scenario"] == 1
+
+
+def _units(N, nb, spread, order, seed=8):
+    """Exponents of power-of-two units, one per variable of every stage, that
+    span 0..spread within each group of eight columns."""
+    i = np.arange(nb) % 8
+    if order == "alternating":
+        e = np.where(i % 2, spread, 0)
+    else:
+        e = np.round(spread * i / 7.0).astype(int)
+        if order == "descending":
+            e = spread - e
+    e = np.tile(e, (N, 1))
+    if order == "shuffled":
+        rng = np.random.default_rng(seed)
+        for k in range(N):
+            for c in range(0, nb, 8):
+                rng.shuffle(e[k, c:c + 8])
+    return e
+
+
+def _in_units(d, e):
+    """The system of d in variables scaled by s = 2^e: S K S x' = S r, x = S x'."""
+    N = d["N"]
+    s = torch.from_numpy(2.0 ** e)
+    f = dict(d, D=s[:, :, None] * d["D"] * s[:, None, :], C=d["C"] * s[0])
+    if N > 1:
+        f["E"] = s[1:, :, None] * d["E"] * s[:-1, None, :]
+    r = d["r"].clone()
+    n0 = d["S"] * N * d["nb"]
+    r[:n0] = (r[:n0].reshape(d["S"], N, d["nb"]) * s).reshape(-1)
+    f["r"] = r
+    return f
+
+
+@pytest.mark.parametrize("order", ["alternating", "ascending", "descending", "shuffled"])
+@pytest.mark.parametrize("spread", [0, 20, 60])
+@pytest.mark.parametrize("S,N,nb,nr", [(2, 6, 12, 4), (2, 6, 16, 5), (1, 7, 24, 8), (1, 5, 32, 11), (1, 5, 48, 16)])
+def test_variables_of_different_units(S, N, nb, nr, spread, order):
+    """The bounds are those of a Cholesky solve whatever the units are: the
+    factor's as above, and for x, with two substitutions of the same sums and
+    |L| |L^T| <= sqrt(K_ii K_jj), |r - K x|_i <= 3 M u sum_j sqrt(K_ii K_jj) |x_j|
+    with M the longest sum of the whole factor (the root's rows gather the
+    nb terms of every tail besides); both sides carry s_i, which divides out."""
+    from oracle import dense
+    d = _gen(S, N, nb, nr)
+    e = _units(N, nb, spread, order)
+    f = _in_units(d, e)
+    x, fac, info = _run(f)
+    assert info["status"] == 0
+    _check_backward_error(f, fac, 1, 2.0 ** -53)
+    n0 = S * N * nb
+    xs = x.astype(np.longdouble)
+    xs[:n0] *= np.tile(2.0 ** e.reshape(-1), S)          # the solution in d's own variables
+    K = dense.assemble_system(d["D"], d["E"], d["C"], d["R"]).astype(np.longdouble)
+    r = d["r"].numpy().astype(np.longdouble)
+    g = np.sqrt(np.diag(K))
+    M = nb * (2 * (N - 1).bit_length() + 1) + S * nb + nr + 1
+    bound = 3 * M * 2.0 ** -53 * g * (g * np.abs(xs)).sum()
+    ratio = float((np.abs(r - K @ xs) / bound).max())
+    assert ratio <= 1.0, ratio
