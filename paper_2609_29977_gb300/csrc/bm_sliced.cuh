@@ -195,14 +195,24 @@ __device__ __forceinline__ double assemble(const float (&c)[ND][4], int t, int E
   // a 2^(81-UP-124) = (m 2^-63) 2^(63-n) 2^(-43-UP); exponents Ea, Eb as 2^(E-1022)
   const int e = (63 - n) - 43 - UP + (Ea - 1022) + (Eb - 1022) + 1023;  // biased exponent of the result
   unsigned rh = (unsigned)(r >> 32) + ((unsigned)(e - 1) << 20), rl = (unsigned)r;
-  if ((unsigned)(e - 1) >= 2045u || a == 0ull) {   // zero, underflow; overflow; inf or NaN in a row
+  if ((unsigned)(e - 1) >= 2046u || a == 0ull) {   // zero, underflow; overflow; inf or NaN in a row
     rl = 0u;
     rh = Ea == kBadRow || Eb == kBadRow ? 0x7ff80000u : a == 0ull || e < 1 ? 0u : 0x7ff00000u;
   }
   return __hiloint2double((int)(rh | ((unsigned)sg & 0x80000000u)), (int)rl);
 }
 
-// Calls out(i, j, value) for the entries (i, j) of A B^T (A: M x K, B: NC x K,
+// Products are put together 2^64 times too large and scaled back (f = 2^-64)
+// by the FP64 instruction that takes them up, so that what is subnormal is
+// rounded and not lost (K near the lower end of the range). Not for rows with
+// entries from 2^448 on, where the scaled product could overflow: K_ii is
+// above 2^896 there, and with any K_jj a product below 2^-1022 does not show.
+// S = 512, N = 128, nb = 24: factor and solve 3836 -> 3862 us, nearly all of
+// it in the updates of rows and the fill; S = 100, N = 160, nb = 16: 605 both.
+__device__ __forceinline__ int up_scale(int E) { return E < 1023 + 448 ? 64 : 0; }
+__device__ __forceinline__ double down_scale(int up) { return __hiloint2double((1023 - up) << 20, 0); }
+
+// Calls out(i, j, v, f) for the entries (i, j), v f, of A B^T (A: M x K, B: NC x K,
 // row-major with strides lda, ldb) that this lane computes; the 16 x 8 tiles
 // are shared by the team's warps. SYRK: B = A, and only tiles that hold
 // entries j <= i; the tiles on the diagonal use A's digits for both sides.
@@ -278,8 +288,9 @@ __device__ __forceinline__ void product(const Team<TEAM> &tm, const double *A, i
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       const int i = mt * 16 + (t >> 1) * 8 + gid, j = nt * 8 + 2 * tig + (t & 1);
-      const double val = assemble<K>(c, t, Ea[t >> 1], (t & 1) ? Eb1 : Eb0);
-      if (i < M && j < NC && (!SYRK || j <= i)) out(i, j, val);
+      const int up = up_scale(Ea[t >> 1]);
+      const double val = assemble<K>(c, t, Ea[t >> 1] + up, (t & 1) ? Eb1 : Eb0);
+      if (i < M && j < NC && (!SYRK || j <= i)) out(i, j, val, down_scale(up));
     }
   }
 }
@@ -291,7 +302,8 @@ __device__ __forceinline__ void team_syrk_sub(const Team<TEAM> &tm, double *sD, 
   for (int w = 0; w < (Y ? 2 : 1); ++w) {
     const double *P = w ? Y : X;
     // every entry is updated by the same lane in both passes
-    product<TEAM, NB, true>(tm, P, NB, NB, P, NB, NB, [&](int i, int j, double v) { sD[i * NB + j] -= v; });
+    product<TEAM, NB, true>(tm, P, NB, NB, P, NB, NB,
+                            [&](int i, int j, double v, double f) { sD[i * NB + j] = fma(-v, f, sD[i * NB + j]); });
   }
 }
 
@@ -299,7 +311,8 @@ __device__ __forceinline__ void team_syrk_sub(const Team<TEAM> &tm, double *sD, 
 template <int TEAM, int NB>
 __device__ __forceinline__ void team_gemm_nt_neg(const Team<TEAM> &tm, double *__restrict__ out, const double *A,
                                                  const double *B) {
-  product<TEAM, NB, false>(tm, A, NB, NB, B, NB, NB, [&](int i, int j, double v) { out[i * NB + j] = -v; });
+  product<TEAM, NB, false>(tm, A, NB, NB, B, NB, NB,
+                           [&](int i, int j, double v, double f) { out[i * NB + j] = -v * f; });
 }
 
 // 1 / d for a positive normal d to about an ulp: an FP32 estimate y of the
@@ -307,11 +320,10 @@ __device__ __forceinline__ void team_gemm_nt_neg(const Team<TEAM> &tm, double *_
 // and the geometric series 1/m = y / (1 - e) cut after e^2, whose rest e^3 is
 // below 2^-63, in FP64 (three dependent FP64 instructions; a library division
 // takes more than twice that), the exponent by integer arithmetic.
-// Subnormal d, and d so large that 1/d is subnormal, take the division.
+// For d between 2^-1022 and 2^1022; d = 2^-1030 would give inf.
 __device__ __forceinline__ double pivot_rcp(double d) {
   const int hi = __double2hiint(d);
   const int e = hi >> 20;
-  if (e < 1 || e > 2044) return 1.0 / d;
   const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(d));   // in [1, 2)
   // the significand's top 23 bits as a float
   const float mf = __uint_as_float(0x3f800000u | ((unsigned)(hi & 0xfffff) << 3) | ((unsigned)__double2loint(d) >> 29));
@@ -343,8 +355,9 @@ __device__ __forceinline__ void tri_fill(TriTable<NB> &t) {
 
 // Cholesky of the block in sA (lower triangle read) by way of M D M^T: the
 // pivots' reciprocals (three FP64 instructions on the critical path) drive
-// the elimination, and the square roots of all pivots are taken at the end,
-// one lane per column. On return the lower triangle holds L, the strict
+// the elimination (those near the ends of the range are scaled first, so that
+// the reciprocal is a normal number), and the square roots of all pivots are
+// taken at the end, one lane per column. On return the lower triangle holds L, the strict
 // upper triangle the transpose of the unit factor M = L diag(L)^-1 (what
 // the tail solves substitute with), and sInv[j] = 1/L_jj. A pivot that is
 // not positive and finite is replaced by 1; returns 1 + its column, 0 if
@@ -355,26 +368,36 @@ __device__ __forceinline__ int team_chol(const Team<TEAM> &tm, double *sA, doubl
 #pragma unroll 1
   for (int j = 0; j < NB - 1; ++j) {
     double d = sA[j * NB + j];
-    if (!pivot_ok(d)) {
-      if (!fail) fail = j + 1;
-      d = 1.0;
-    }
-    const double r = pivot_rcp(d);
     const int m = NB - 1 - j, ne = m * (m + 1) / 2;
-    for (int i = j + 1 + tm.lane; i < NB; i += TEAM) sA[j * NB + i] = sA[i * NB + j] * r;
-    if (TEAM == 32) {
-      tm.sync();
-      for (int e = tm.lane; e < ne; e += TEAM) {
-        const int ab = tri.at[e], i = j + 1 + (ab & 255), k = j + 1 + (ab >> 8);
-        sA[i * NB + k] = fma(-sA[j * NB + i], sA[k * NB + j], sA[i * NB + k]);
+    // unit(a) = a / d
+    auto eliminate = [&](auto unit) {
+      for (int i = j + 1 + tm.lane; i < NB; i += TEAM) sA[j * NB + i] = unit(sA[i * NB + j]);
+      if (TEAM == 32) {
+        tm.sync();
+        for (int e = tm.lane; e < ne; e += TEAM) {
+          const int ab = tri.at[e], i = j + 1 + (ab & 255), k = j + 1 + (ab >> 8);
+          sA[i * NB + k] = fma(-sA[j * NB + i], sA[k * NB + j], sA[i * NB + k]);
+        }
+      } else {
+        // several warps: each element scales its own row entry again (the
+        // same product) instead of waiting for the column at a barrier
+        for (int e = tm.lane; e < ne; e += TEAM) {
+          const int ab = tri.at[e], i = j + 1 + (ab & 255), k = j + 1 + (ab >> 8);
+          sA[i * NB + k] = fma(-unit(sA[i * NB + j]), sA[k * NB + j], sA[i * NB + k]);
+        }
       }
-    } else {
-      // several warps: each element scales its own row entry again (the
-      // same product) instead of waiting for the column at a barrier
-      for (int e = tm.lane; e < ne; e += TEAM) {
-        const int ab = tri.at[e], i = j + 1 + (ab & 255), k = j + 1 + (ab >> 8);
-        sA[i * NB + k] = fma(-(sA[i * NB + j] * r), sA[k * NB + j], sA[i * NB + k]);
+    };
+    // (the same for the whole team)
+    if ((unsigned)(__double2hiint(d) - (64 << 20)) < (1900u << 20)) {
+      const double r = pivot_rcp(d);
+      eliminate([&](double a) { return a * r; });
+    } else {   // not positive and finite, or 1/d could overflow or be subnormal
+      if (!pivot_ok(d)) {
+        if (!fail) fail = j + 1;
+        d = 1.0;
       }
+      const double t = d < 1.0 ? 0x1p64 : 0x1p-64, r = pivot_rcp(d * t);
+      eliminate([&](double a) { return (a * t) * r; });
     }
     tm.sync();
   }
@@ -508,8 +531,10 @@ __device__ __forceinline__ void trsm_panel(double (&x)[2][NB / 8][2], const doub
     }
     const int Eb0 = __shfl_sync(0xffffffffu, Eb, 8 * tig), Eb1 = __shfl_sync(0xffffffffu, Eb, 8 * tig + 4);
 #pragma unroll
-    for (int t = 0; t < 4; ++t)
-      x[t >> 1][P][t & 1] -= assemble<c0>(c, t, t >> 1 ? E1 : E0, (t & 1) ? Eb1 : Eb0);
+    for (int t = 0; t < 4; ++t) {
+      const int E = t >> 1 ? E1 : E0, up = up_scale(E);
+      x[t >> 1][P][t & 1] = fma(-assemble<c0>(c, t, E + up, (t & 1) ? Eb1 : Eb0), down_scale(up), x[t >> 1][P][t & 1]);
+    }
   }
   double b[1][2];
   load_rows<8>(b, sA + c0 * NB + c0, NB, gid, 8);
@@ -526,7 +551,8 @@ __device__ __forceinline__ void trsm_panel(double (&x)[2][NB / 8][2], const doub
   accumulate8(c, a0, a1, bd);
   const int Eb0 = __shfl_sync(0xffffffffu, Eb, 8 * tig), Eb1 = __shfl_sync(0xffffffffu, Eb, 8 * tig + 4);
 #pragma unroll
-  for (int t = 0; t < 4; ++t) x[t >> 1][P][t & 1] = assemble<8>(c, t, t >> 1 ? E1 : E0, (t & 1) ? Eb1 : Eb0);
+  for (int t = 0; t < 4; ++t)   // (entries of X: against sqrt(K_ii) > 2^-538 a subnormal one does not show)
+    x[t >> 1][P][t & 1] = assemble<8>(c, t, t >> 1 ? E1 : E0, (t & 1) ? Eb1 : Eb0);
   if constexpr (c0 + 8 < NB) trsm_panel<NB, P + 1>(x, sA, inv);
 }
 

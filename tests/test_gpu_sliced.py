@@ -197,3 +197,71 @@ def test_variables_of_different_units(S, N, nb, nr, spread, order):
     bound = 3 * M * 2.0 ** -53 * g * (g * np.abs(xs)).sum()
     ratio = float((np.abs(r - K @ xs) / bound).max())
     assert ratio <= 1.0, ratio
+
+
+def _check_backward_error_at_the_edge(d, fac):
+    """As _check_backward_error (barrier-free systems, u = 2^-53), with the
+    subnormal range's absolute rounding: half of 2^-1074 for each of an
+    entry's nb (2 levels + 1) operations."""
+    S, N, nb = d["S"], d["N"], d["nb"]
+    m = nb * (2 * (N - 1).bit_length() + 1)
+    for s in range(S):
+        from oracle import dense
+        K = dense.assemble_tail(d["D"][s], d["E"][s]).astype(np.longdouble)
+        L = np.zeros_like(K)
+        at = lambda p: slice((N - p) * nb, (N - p + 1) * nb)  # noqa: E731  (stage N + 1 - p)
+        for p in range(1, N + 1):
+            k = N - p
+            L[at(p), at(p)] = np.tril(fac["Ld"][s, k])
+            if p < N:
+                h = p & -p
+                L[at(p + h if p + h <= N - 1 else N), at(p)] = fac["Lr"][s, k]
+                if p > h:
+                    L[at(p - h), at(p)] = fac["Ll"][s, k]
+        g = np.sqrt(np.diag(K))
+        bound = (m + 1) * (np.longdouble(2.0) ** -53 * np.outer(g, g) + np.longdouble(2.0) ** -1075)
+        ratio = float((np.abs(K - L @ L.T) / bound).max())
+        assert ratio <= 1.0, ratio
+
+
+@pytest.mark.parametrize("S,N,nb,nr", [(2, 6, 12, 4), (2, 6, 16, 5), (1, 7, 24, 8), (1, 5, 32, 11), (1, 5, 48, 16)])
+@pytest.mark.parametrize("end", ["subnormal", "largest"])
+def test_scales_at_the_ends_of_the_range(S, N, nb, nr, end):
+    """K scaled so far down that its entries and pivots are subnormal (below
+    2^-1024, where 1/d overflows), or so far up that the largest lie in the
+    last binade."""
+    w = bmgen.Workload("t", S, N, nb, nr, shared_A=True)
+    d = bmgen.generate(w, seed=4)
+    top = max(float(d[k].abs().max()) for k in "DECR")
+    k = -1033 - int(np.ceil(np.log2(top))) if end == "subnormal" else 1024 - int(np.floor(np.log2(top))) - 1
+    # in two steps, so that no factor is itself out of range; r as it is: the
+    # solution scales by 2^-k, out of range at the lower end, so r goes along
+    f = lambda t: t * 2.0 ** (k // 2) * 2.0 ** (k - k // 2)  # noqa: E731
+    e = dict(d, D=f(d["D"]), E=f(d["E"]), C=f(d["C"]), R=f(d["R"]), r=f(d["r"]))
+    x, fac, info = _run(e)
+    assert info["status"] == 0
+    _check_backward_error_at_the_edge(e, fac)
+    assert np.isfinite(x).all()
+
+
+@pytest.mark.parametrize("nb", [12, 16, 24, 32, 48])
+@pytest.mark.parametrize("col", [0, 5, -1])
+def test_decoupled_variable_with_a_subnormal_pivot(nb, col):
+    """A variable that nothing couples to, with a diagonal entry whose
+    reciprocal overflows: its factor entry is the square root, the others
+    are those of the system without it, and x_c = r_c / d."""
+    S, N, nr, s, k = 2, 6, 3, 1, 2
+    d = _gen(S, N, nb, nr)
+    d = {q: (v.clone() if isinstance(v, torch.Tensor) else v) for q, v in d.items()}
+    D, E = d["D"], d["E"]
+    D[s, k, col, :] = 0.0
+    D[s, k, :, col] = 0.0
+    D[s, k, col, col] = 2.0 ** -1030
+    E[s, k - 1, col, :] = 0.0
+    E[s, k, :, col] = 0.0
+    d["r"][((s * N + k) * nb) + col % nb] = 3.0 * 2.0 ** -1030
+    x, fac, info = _run(d)
+    assert info["status"] == 0
+    _check_backward_error(d, fac, 1, 2.0 ** -53)
+    assert fac["Ld"][s, k, col, col] == 2.0 ** -515
+    assert x[((s * N + k) * nb) + col % nb] == 3.0
