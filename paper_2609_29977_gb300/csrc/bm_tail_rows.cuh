@@ -662,11 +662,29 @@ __global__ void __launch_bounds__(128, 4) k_level_rows(TailView<T> v, int lvl) {
   pdl_trigger();
 }
 
-// Top levels lvl0..Lc-1 and x_1 of one tail per CTA (four teams). Four CTAs
-// per SM: left to itself the compiler takes 255 registers for nb = 24, two
-// CTAs fit and 512 tails need two waves (S = 512, N = 128: 154 -> 109 us).
+// Teams of the top kernel's CTA. Its levels have at most four positions each;
+// with many tails the further teams idle in most of them and cost the
+// registers and shared memory of other tails.
+// nb = 24 and 32 take 255 registers (at 128, for four CTAs of four teams per
+// SM, they spill 300 to 700 bytes, whatever S is). So that all tails stay on
+// the SMs at once there are four teams up to two tails per SM (304), two up to
+// four (608), one beyond. Factor, us, four teams at 128 registers -> this
+// rule: nb = 24: S = 150, N = 6 109 -> 91; S = 304, N = 64 367 -> 352; S = 512, N = 6
+// 144 -> 109, N = 128 882 -> 867; S = 609, N = 20 334 -> 252; nb = 32: S = 4, N = 8
+// 171 -> 150; S = 304, N = 8 258 -> 212; S = 512, N = 6 397 -> 222; S = 1000, N = 12
+// 710 -> 558. Slower between three tails per SM and more levels: nb = 32,
+// S = 400, N = 20 412 -> 445, N = 64 848 -> 867 (four teams uncapped: S = 440,
+// N = 20 434 -> 510). Two teams from S = 153 on: S = 153, N = 8 92 -> 101 (nb = 24).
+template <int NB>
+inline int top_teams(int S) {
+  return NB <= 16 || S <= 2 * 152 ? 4 : S <= 4 * 152 ? 2 : 1;
+}
+
+// Top levels lvl0..Lc-1 and x_1 of one tail per CTA. Four CTAs per SM for the
+// smaller blocks, which fit 128 registers: left to itself the compiler takes
+// up to 254 (factor of S = 1000, N = 12, nb = 16: 136 us, uncapped 161).
 template <typename T, int NB>
-__global__ void __launch_bounds__(128, 4) k_top_rows(TailView<T> v, int lvl0) {
+__global__ void __launch_bounds__(128, NB <= 16 ? 4 : 1) k_top_rows(TailView<T> v, int lvl0) {
   constexpr int TS = Cfg<NB>::TS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int team = threadIdx.x / TS, lane = threadIdx.x % TS, teams = blockDim.x / TS;
@@ -707,7 +725,7 @@ void launch_tail_rows(const TailView<T> &v, cudaStream_t st) {
     const long blocks = (tasks + tpc - 1) / tpc;
     launch_pdl(k_level_rows<T, NB>, (unsigned)blocks, 128, (size_t)tpc * Cfg<NB>::SM * sizeof(T), st, v, l);
   }
-  const int teams = 4;
+  const int teams = top_teams<NB>(v.S);
   size_t smem = (size_t)teams * Cfg<NB>::SM * sizeof(T);
   const size_t x1b = x1_rows_bytes<T, NB>(v.nr);
   if (x1b > smem) smem = x1b;

@@ -68,6 +68,26 @@ def test_substitutions_and_residuals_give_the_batched_forms_bits(S, N, nb, tmp_p
     assert torch.equal(x, xb)
 
 
+# the top levels' CTAs have fewer teams from three and from five tails per SM
+# on: the first and last tails of a system against the same tails alone
+@pytest.mark.parametrize("nb", [24, 32])
+@pytest.mark.parametrize("S,N", [(305, 2), (305, 5), (608, 9), (609, 4), (609, 7)])
+def test_top_levels_with_fewer_teams_give_the_same_factor(S, N, nb):
+    import paper_2609_29977_gb300 as bm
+    d = _system(S, N, nb)
+    keep = torch.tensor([0, 1, S - 2, S - 1], device="cuda")
+    few = {k: d[k][keep].contiguous() for k in ("D", "E", "C")}
+    out = []
+    for q, D, E, C in ((S, d["D"], d["E"], d["C"]), (4, few["D"], few["E"], few["C"])):
+        solver = bm.BranchKKTSolver(q, N, nb, d["nr"], precision=bm.BM_PREC_FP32_IR)
+        solver.factor(D, E, C, d["R"])
+        assert solver.query()["status"] == 0
+        out.append(solver.export_factor())
+        solver.close()
+    for k in ("Ld", "Ll", "Lr", "F"):
+        assert torch.equal(out[0][k][keep], out[1][k]), k
+
+
 # arrays eight bytes off a 16-byte boundary, which a batch has always taken
 @pytest.mark.parametrize("nb", [4, 6, 24, 48])
 def test_batch_takes_arrays_eight_bytes_off(nb, tmp_path, monkeypatch):
