@@ -53,9 +53,11 @@ __host__ __device__ inline int xt_blocks(int S, int N, int nb, int nr) {
 // iter >= 0: a directly launched iteration; iter < 0: the body of a graph
 // loop, whose iteration index is read from the control block and whose
 // condition handle is cond.
-template <int NB>
-__global__ void __launch_bounds__(SubCfg<NB>::THREADS, 4) k_mixed_fwd(MixedState m, const double *__restrict__ r, double *x, int iter,
-                                                    int CS, cudaGraphConditionalHandle cond) {
+// MINB: CTAs per SM (five_ctas).
+template <int NB, int MINB>
+__global__ void __launch_bounds__(SubCfg<NB>::THREADS, MINB) k_mixed_fwd(MixedState m, const double *__restrict__ r,
+                                                                         double *x, int iter, int CS,
+                                                                         cudaGraphConditionalHandle cond) {
   // the tail's part, then the root step
   constexpr int F = SubCfg<NB>::floats(SubCfg<NB>::THREADS) / 2, R = 64 * 64 + 64 + 64;
   __shared__ __align__(16) double sbuf[F > R ? F : R];
@@ -69,8 +71,8 @@ __global__ void __launch_bounds__(SubCfg<NB>::THREADS, 4) k_mixed_fwd(MixedState
   if (last_cta(&m.tickets[2], gridDim.x)) root_step<NB>(m, rhs, x, it, sbuf, coupled(m) ? xt_blocks(m.S, m.N, NB, m.nr) : m.S);
 }
 
-template <int NB>
-__global__ void __launch_bounds__(SubCfg<NB>::THREADS, 4) k_mixed_bwd(MixedState m, double *x, int iter, int CS) {
+template <int NB, int MINB>
+__global__ void __launch_bounds__(SubCfg<NB>::THREADS, MINB) k_mixed_bwd(MixedState m, double *x, int iter, int CS) {
   __shared__ __align__(16) float sbuf[SubCfg<NB>::floats(SubCfg<NB>::THREADS)];
   pdl_wait();
   if (ir_done(m.ctl)) return;
@@ -397,6 +399,13 @@ void launch_plain(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t 
   cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// CTAs per SM of the substitutions: four (64 registers), or five (48, some
+// spilling) where all CTAs then run in fewer waves. Solve, us, four -> five: S = 700,
+// N = 24: nb = 4 187 -> 154, nb = 8 221 -> 185, nb = 16 289 -> 240, nb = 32 654 -> 568;
+// S = 2000: 320 -> 292, 459 -> 435, 981 -> 949, 1435 -> 1426. With as many waves
+// five are slower: S = 512, N = 128, nb = 16 455 -> 483, S = 1000, N = 60 788 -> 855.
+inline bool five_ctas(long ctas) { return (ctas + 5 * 152 - 1) / (5 * 152) < (ctas + 4 * 152 - 1) / (4 * 152); }
+
 // One iteration (iter >= 0), or the body of the graph loop (iter = -1).
 template <int NB>
 void launch_iteration(const MixedState &m, const double *r, double *x, int iter, int max_iter, double tol,
@@ -408,8 +417,12 @@ void launch_iteration(const MixedState &m, const double *r, double *x, int iter,
     launch_plain(k_mixed_bwd_chain<NB>, (unsigned)m.S, 256, vec, pdl, st, m, x, iter);
   } else {
     const unsigned grid = (unsigned)(m.S * CS);
-    launch_cluster(k_mixed_fwd<NB>, grid, SubCfg<NB>::THREADS, CS, pdl, st, m, r, x, iter, CS, cond);
-    launch_cluster(k_mixed_bwd<NB>, grid, SubCfg<NB>::THREADS, CS, pdl, st, m, x, iter, CS);
+    constexpr int MORE = SubCfg<NB>::PAIR ? 4 : 5;
+    const bool more = five_ctas((long)m.S * CS);
+    launch_cluster(more ? k_mixed_fwd<NB, MORE> : k_mixed_fwd<NB, 4>, grid, SubCfg<NB>::THREADS, CS, pdl, st, m, r, x,
+                   iter, CS, cond);
+    launch_cluster(more ? k_mixed_bwd<NB, MORE> : k_mixed_bwd<NB, 4>, grid, SubCfg<NB>::THREADS, CS, pdl, st, m, x, iter,
+                   CS);
   }
   const int blocks = xt_blocks(m.S, m.N, NB, m.nr);
   launch_plain(k_mixed_residual<NB>, (unsigned)blocks, 256, FFCfg<NB>::bytes, pdl, st, m, r, (const double *)x, iter, max_iter, tol,

@@ -68,6 +68,12 @@ def test_substitutions_and_residuals_give_the_batched_forms_bits(S, N, nb, tmp_p
     assert torch.equal(x, xb)
 
 
+# five CTAs per SM where that saves a wave, four beside it
+@pytest.mark.parametrize("S,N,nb", [(608, 3, 4), (609, 3, 4), (760, 9, 6), (761, 2, 12), (700, 5, 24), (1217, 2, 6)])
+def test_substitutions_with_more_ctas_give_the_batched_forms_bits(S, N, nb, tmp_path, monkeypatch):
+    test_substitutions_and_residuals_give_the_batched_forms_bits(S, N, nb, tmp_path, monkeypatch)
+
+
 # the top levels' CTAs have fewer teams from three and from five tails per SM
 # on: the first and last tails of a system against the same tails alone
 @pytest.mark.parametrize("nb", [24, 32])
