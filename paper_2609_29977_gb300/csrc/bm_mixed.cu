@@ -80,11 +80,9 @@ __global__ void __launch_bounds__(SubCfg<NB>::THREADS, MINB) k_mixed_bwd(MixedSt
 }
 
 // The same two kernels for few tails (chain_applies): one CTA per tail.
-template <int NB>
-__global__ void __launch_bounds__(256, ChainCfg<NB>::CTAS) k_mixed_fwd_chain(MixedState m,
-                                                                             const double *__restrict__ r, double *x,
-                                                                             int iter,
-                                                                             cudaGraphConditionalHandle cond) {
+template <int NB, int CTAS>
+__global__ void __launch_bounds__(256, CTAS) k_mixed_fwd_chain(MixedState m, const double *__restrict__ r, double *x,
+                                                               int iter, cudaGraphConditionalHandle cond) {
   extern __shared__ __align__(16) double sV[];   // the tail's vectors, then the root step
   __shared__ float sY[MCfg<NB>::TEAMS][NB];
   pdl_wait();
@@ -96,8 +94,8 @@ __global__ void __launch_bounds__(256, ChainCfg<NB>::CTAS) k_mixed_fwd_chain(Mix
   if (last_cta(&m.tickets[2], gridDim.x)) root_step<NB>(m, rhs, x, it, sV, coupled(m) ? xt_blocks(m.S, m.N, NB, m.nr) : m.S);
 }
 
-template <int NB>
-__global__ void __launch_bounds__(256, ChainCfg<NB>::CTAS) k_mixed_bwd_chain(MixedState m, double *x, int iter) {
+template <int NB, int CTAS>
+__global__ void __launch_bounds__(256, CTAS) k_mixed_bwd_chain(MixedState m, double *x, int iter) {
   extern __shared__ __align__(16) double sV[];
   __shared__ float sX[MCfg<NB>::TEAMS][NB];
   pdl_wait();
@@ -413,8 +411,12 @@ void launch_iteration(const MixedState &m, const double *r, double *x, int iter,
   const int CS = pick_cluster(m.S);
   if (chain_applies<NB>(m.S, m.N, CS)) {
     const size_t vec = (size_t)m.N * NB * sizeof(float), root = ((size_t)m.nr * m.nr + m.nr) * sizeof(double);
-    launch_plain(k_mixed_fwd_chain<NB>, (unsigned)m.S, 256, vec > root ? vec : root, pdl, st, m, r, x, iter, cond);
-    launch_plain(k_mixed_bwd_chain<NB>, (unsigned)m.S, 256, vec, pdl, st, m, x, iter);
+    constexpr int ALL = ChainCfg<NB>::CTAS, FEW = ChainCfg<NB>::FEW;
+    const bool few = m.S <= 152 * FEW;
+    launch_plain(few ? k_mixed_fwd_chain<NB, FEW> : k_mixed_fwd_chain<NB, ALL>, (unsigned)m.S, 256,
+                 vec > root ? vec : root, pdl, st, m, r, x, iter, cond);
+    launch_plain(few ? k_mixed_bwd_chain<NB, FEW> : k_mixed_bwd_chain<NB, ALL>, (unsigned)m.S, 256, vec, pdl, st, m, x,
+                 iter);
   } else {
     const unsigned grid = (unsigned)(m.S * CS);
     constexpr int MORE = SubCfg<NB>::PAIR ? 4 : 5;
@@ -567,6 +569,14 @@ bool mixed_ff_residual(double tol, unsigned flags) {
 bool mixed_ffres(const MixedState *m) { return m->ffres != 0; }
 
 
+template <int NB, int CTAS>
+static cudaError_t prepare_chain() {
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_mixed_fwd_chain<NB, CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_mixed_bwd_chain<NB, CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+}
+
 cudaError_t mixed_prepare(int nb, int nr) {
   (void)nr;
   if (!tail_nb_supported(nb)) return cudaErrorInvalidValue;
@@ -582,10 +592,8 @@ cudaError_t mixed_prepare(int nb, int nr) {
     e = cudaFuncSetAttribute(k_mixed_residual<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);    \
   if (e == cudaSuccess)                                                                                       \
     e = cudaFuncSetAttribute(k_residual_out<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);      \
-  if (e == cudaSuccess)                                                                                       \
-    e = cudaFuncSetAttribute(k_mixed_fwd_chain<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);   \
-  if (e == cudaSuccess)                                                                                       \
-    e = cudaFuncSetAttribute(k_mixed_bwd_chain<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+  if (e == cudaSuccess) e = prepare_chain<n, ChainCfg<n>::CTAS>();                                            \
+  if (e == cudaSuccess && ChainCfg<n>::FEW != ChainCfg<n>::CTAS) e = prepare_chain<n, ChainCfg<n>::FEW>();
   BM_TAIL_NB_LIST(X)
 #undef X
   if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;

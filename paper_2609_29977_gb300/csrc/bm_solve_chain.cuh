@@ -26,6 +26,10 @@ struct ChainCfg {
   static constexpr int TS = MCfg<NB>::TS, TEAMS = MCfg<NB>::TEAMS;
   // CTAs per SM that the registers allow (three rows of the factor per lane)
   static constexpr int CTAS = NB <= 32 ? 2 : 1;
+  // for nb = 32 only with spilling (128 registers of 155 and 201): up to 152
+  // tails get one CTA per SM instead. Solve, us: S = 4, N = 8 138 -> 130;
+  // S = 64, N = 12 155 -> 146; S = 150, N = 64 410 -> 380
+  static constexpr int FEW = NB == 32 ? 1 : CTAS;
   static constexpr size_t MAX_VEC = 96 * 1024;   // bytes of one tail's vectors
 };
 
@@ -48,11 +52,12 @@ inline int chain_rounds(int N) {
 //   S=140 N=100 nb=48 (42, 1) 1123 -> 913  S=280 N=100 nb=12 (18, 1) 379 -> 302
 //   S=8 N=64 nb=24 (15, 8) 156 -> 160      S=20 N=200 nb=12 (24, 4) 168 -> 165
 //   S=10 N=128 nb=24 (26, 8) 171 -> 225    S=40 N=60 nb=48 (25, 2) 411 -> 465
-//   S=30 N=250 nb=32 (49, 4) 648 -> 1027
+//   S=30 N=250 nb=32 (49, 4) 648 -> 1027   S=4 N=30 nb=32 (8, 8) 177 -> 166
+//   S=4 N=40 nb=32 (12, 8) 189 -> 193
 template <int NB>
 inline bool chain_applies(int S, int N, int cluster) {
   return S <= 152 * ChainCfg<NB>::CTAS && (size_t)N * NB * sizeof(float) <= ChainCfg<NB>::MAX_VEC &&
-         (cluster == 1 || chain_rounds<NB>(N) <= 12);
+         (cluster == 1 || chain_rounds<NB>(N) <= (NB < 32 ? 12 : 11));
 }
 
 struct ChainItem {

@@ -74,6 +74,30 @@ def test_substitutions_with_more_ctas_give_the_batched_forms_bits(S, N, nb, tmp_
     test_substitutions_and_residuals_give_the_batched_forms_bits(S, N, nb, tmp_path, monkeypatch)
 
 
+# nb = 32, which the batch does not take: one CTA per SM and per tail, two, and
+# the cluster kernels. The tails beyond the first 152 do not couple to the root,
+# and the tolerance stops after the first solve, before any sum over all rows.
+@pytest.mark.parametrize("N", [1, 2, 9, 33])
+def test_forms_for_few_tails_of_wide_blocks_give_the_same_bits(N):
+    import paper_2609_29977_gb300 as bm
+    S, nb = 152, 32
+    d = _system(S, N, nb)
+    n, nr = S * N * nb, d["nr"]
+    out = []
+    for q in (S, S + 1, 2 * S, 2 * S + 1):
+        m = torch.arange(q, device="cuda") % S
+        D, E, C = (d[k][m].contiguous() for k in ("D", "E", "C"))
+        C[S:] = 0.0
+        r = torch.cat([d["r"][:n].reshape(S, -1)[m].reshape(-1), d["r"][n:]])
+        solver = bm.BranchKKTSolver(q, N, nb, nr, precision=bm.BM_PREC_FP32_IR, tol=1e-2, flags=bm.BM_FLAG_COUPLING_FP32)
+        solver.factor(D, E, C, d["R"])
+        x, info = solver.solve(r), solver.query()
+        solver.close()
+        assert info["status"] == 0 and info["iters"] == 0
+        out.append(torch.cat([x[:n], x[-nr:]]))
+    assert all(torch.equal(o, out[0]) for o in out)
+
+
 # the top levels' CTAs have fewer teams from three and from five tails per SM
 # on: the first and last tails of a system against the same tails alone
 @pytest.mark.parametrize("nb", [24, 32])
