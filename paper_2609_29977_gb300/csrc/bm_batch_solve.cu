@@ -65,7 +65,15 @@ __global__ void __launch_bounds__(256, 3) k_batch_bwd(const BInst *inst, const B
   }
 }
 
-__global__ void __launch_bounds__(256, 3) k_batch_res(const BInst *inst, const BTail *tails, const double *const *rp,
+// MINB: CTAs per SM, three (80 registers), or four (64, some spilling) where
+// all tails then run in fewer waves. 16 systems of 30 tails, N = 60, solve, us,
+// three -> four: nb = 6 478 -> 464, 12 740 -> 710, 24 1417 -> 1320, 48 3987 -> 3641;
+// with as many waves (8 systems of 100 tails, N = 100) 24 2809 -> 3015, 48
+// 7504 -> 8321.
+inline bool four_ctas(long ctas) { return (ctas + 4 * 152 - 1) / (4 * 152) < (ctas + 3 * 152 - 1) / (3 * 152); }
+
+template <int MINB>
+__global__ void __launch_bounds__(256, MINB) k_batch_res(const BInst *inst, const BTail *tails, const double *const *rp,
                                                       double *const *xp, int iter, int max_iter, double tol) {
   __shared__ double sbuf[8 * ResCfg<48>::WARP];
   const BTail t = tails[blockIdx.x];
@@ -95,7 +103,8 @@ void batch_launch_solve_iteration(const BInst *inst, const BTail *tails, int nta
                                   double *const *x, int iter, int max_iter, double tol, cudaStream_t st) {
   launch_pdl(k_batch_fwd, (unsigned)ntails, 256, 0, st, inst, tails, r, x, iter);
   launch_pdl(k_batch_bwd, (unsigned)ntails, 256, 0, st, inst, tails, x, iter);
-  launch_pdl(k_batch_res, (unsigned)ntails, 256, 0, st, inst, tails, r, x, iter, max_iter, tol);
+  launch_pdl(four_ctas(ntails) ? k_batch_res<4> : k_batch_res<3>, (unsigned)ntails, 256, 0, st, inst, tails, r, x, iter,
+             max_iter, tol);
 }
 
 }  // namespace bm

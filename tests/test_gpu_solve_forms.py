@@ -74,6 +74,12 @@ def test_substitutions_with_more_ctas_give_the_batched_forms_bits(S, N, nb, tmp_
     test_substitutions_and_residuals_give_the_batched_forms_bits(S, N, nb, tmp_path, monkeypatch)
 
 
+# the batched residual with four CTAs per SM (457 to 608 tails), three beside it
+@pytest.mark.parametrize("S,N,nb", [(456, 3, 6), (457, 5, 24), (608, 3, 48), (609, 3, 24), (457, 2, 12)])
+def test_batched_residual_with_more_ctas_gives_the_same_bits(S, N, nb, tmp_path, monkeypatch):
+    test_substitutions_and_residuals_give_the_batched_forms_bits(S, N, nb, tmp_path, monkeypatch)
+
+
 # nb = 32, which the batch does not take: one CTA per SM and per tail, two, and
 # the cluster kernels. The tails beyond the first 152 do not couple to the root,
 # and the tolerance stops after the first solve, before any sum over all rows.
