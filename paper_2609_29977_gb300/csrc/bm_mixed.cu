@@ -109,10 +109,13 @@ __global__ void __launch_bounds__(256, CTAS) k_mixed_bwd_chain(MixedState m, dou
 // the root rows. With refined coupling columns each CTA then leaves its part
 // of the next correction's root term X^T rho in tb. The last CTA applies
 // the stopping test.
-template <int NB>
-__global__ void __launch_bounds__(256, FFCfg<NB>::STAGED ? 3 : 5) k_mixed_residual(MixedState m, const double *__restrict__ r,
-                                                         const double *__restrict__ x, int iter, int max_iter,
-                                                         double tol, cudaGraphConditionalHandle cond) {
+// FF: the handle computes float-float residuals (m.ffres); a handle of FP64
+// residuals gets a kernel without the float-float form's registers and shared
+// memory (nb = 48: 80 registers and 57 KB, three CTAs per SM of five).
+template <int NB, bool FF>
+__global__ void __launch_bounds__(256, FF && FFCfg<NB>::STAGED ? 3 : 5)
+    k_mixed_residual(MixedState m, const double *__restrict__ r, const double *__restrict__ x, int iter, int max_iter,
+                     double tol, cudaGraphConditionalHandle cond) {
   extern __shared__ __align__(16) float sE[];
   __shared__ unsigned sroot;
   pdl_wait();
@@ -121,10 +124,10 @@ __global__ void __launch_bounds__(256, FFCfg<NB>::STAGED ? 3 : 5) k_mixed_residu
   const long nrow = (long)m.S * m.N * NB;
   // float-float unless the handle computes FP64 residuals or an entry of K
   // or x left the float-float range (uniform over the grid)
-  const bool ffr = m.ffres && __ldcg(&m.status->ffbad) == 0;
+  const bool ffr = FF && __ldcg(&m.status->ffbad) == 0;
   float om = 0.0f;
   if (ffr) {
-    om = residual_ff<NB>(m, r, x, sE);
+    if constexpr (FF) om = residual_ff<NB>(m, r, x, sE);
   } else {
     for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < nrow; e += (long)gridDim.x * blockDim.x) {
       const long br = e / NB;
@@ -299,20 +302,24 @@ __global__ void __launch_bounds__(256) k_x_split(MixedState m, const double *__r
 
 // rho = r - K x with the refinement's arithmetic (bm_residual): m.rho is
 // the caller's array.
-template <int NB>
-__global__ void __launch_bounds__(256) k_residual_out(MixedState m, const double *__restrict__ r,
-                                                       const double *__restrict__ x) {
+// FF as in k_mixed_residual. One kernel for both residuals took 165 registers
+// for nb = 48, one CTA per SM. S = 512, N = 128, us, that kernel -> this one:
+// float-float nb = 48 1000 -> 617, nb = 32 319 -> 313; FP64 nb = 48 1273 -> 1043,
+// nb = 24 255 -> 227.
+template <int NB, bool FF>
+__global__ void __launch_bounds__(256, !FF ? 0 : FFCfg<NB>::STAGED ? 3 : NB == 32 ? 4 : 0)
+    k_residual_out(MixedState m, const double *__restrict__ r, const double *__restrict__ x) {
   extern __shared__ __align__(16) float sE[];
   const long nrow = (long)m.S * m.N * NB;
-  const bool ffr = m.ffres && __ldcg(&m.status->ffbad) == 0;
+  const bool ffr = FF && __ldcg(&m.status->ffbad) == 0;
   if (ffr) {
-    residual_ff<NB>(m, r, x, sE);
+    if constexpr (FF) residual_ff<NB>(m, r, x, sE);
   } else {
     for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < nrow; e += (long)gridDim.x * blockDim.x) {
       const long br = e / NB;
       const int i = (int)(e - br * NB);
       const int s = (int)(br / m.N), k = (int)(br - (long)s * m.N);
-      residual_row<NB>(m, r, x, s, k, i);
+      residual_row<NB, NB == 48 || (NB == 24 && !FF)>(m, r, x, s, k, i);
     }
   }
   for (int c = blockIdx.x; c < m.nr; c += gridDim.x) residual_root_row(m, r, x, NB, c);
@@ -427,8 +434,12 @@ void launch_iteration(const MixedState &m, const double *r, double *x, int iter,
                    CS);
   }
   const int blocks = xt_blocks(m.S, m.N, NB, m.nr);
-  launch_plain(k_mixed_residual<NB>, (unsigned)blocks, 256, FFCfg<NB>::bytes, pdl, st, m, r, (const double *)x, iter, max_iter, tol,
-               cond);
+  if (m.ffres)
+    launch_plain(k_mixed_residual<NB, true>, (unsigned)blocks, 256, FFCfg<NB>::bytes, pdl, st, m, r, (const double *)x,
+                 iter, max_iter, tol, cond);
+  else
+    launch_plain(k_mixed_residual<NB, false>, (unsigned)blocks, 256, 0, pdl, st, m, r, (const double *)x, iter, max_iter,
+                 tol, cond);
 }
 
 // Adds the refinement loop to the graph being captured on st: a conditional
@@ -589,9 +600,9 @@ cudaError_t mixed_prepare(int nb, int nr) {
   cudaError_t e = tail_factor_prepare();
 #define X(n)                                                                                                  \
   if (e == cudaSuccess)                                                                                       \
-    e = cudaFuncSetAttribute(k_mixed_residual<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);    \
+    e = cudaFuncSetAttribute(k_mixed_residual<n, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024); \
   if (e == cudaSuccess)                                                                                       \
-    e = cudaFuncSetAttribute(k_residual_out<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);      \
+    e = cudaFuncSetAttribute(k_residual_out<n, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024); \
   if (e == cudaSuccess) e = prepare_chain<n, ChainCfg<n>::CTAS>();                                            \
   if (e == cudaSuccess && ChainCfg<n>::FEW != ChainCfg<n>::CTAS) e = prepare_chain<n, ChainCfg<n>::FEW>();
   BM_TAIL_NB_LIST(X)
@@ -799,7 +810,10 @@ void mixed_launch_residual(MixedState *m, const double *r, const double *x, doub
   switch (m->nb) {
 #define X(n)                                                        \
   case n:                                                           \
-    k_residual_out<n><<<(unsigned)blocks, 256, FFCfg<n>::bytes, st>>>(c, r, x); \
+    if (c.ffres)                                                    \
+      k_residual_out<n, true><<<(unsigned)blocks, 256, FFCfg<n>::bytes, st>>>(c, r, x); \
+    else                                                            \
+      k_residual_out<n, false><<<(unsigned)blocks, 256, 0, st>>>(c, r, x); \
     break;
     BM_TAIL_NB_LIST(X)
 #undef X

@@ -770,8 +770,10 @@ __device__ __forceinline__ float omega_of(double rho, float w) {
 }
 
 // Row i of block row (s, k) of the residual: rho_i = r_i - (K x)_i (stored
-// in m.rho) and its omega_i. Lanes i >= NB must not call it.
-template <int NB>
+// in m.rho) and its omega_i. Lanes i >= NB must not call it. LEAN: fewer loads
+// in flight; where omega is not used the compiler holds all columns of a block
+// at once otherwise (128 registers for nb = 48, 80 for 24).
+template <int NB, bool LEAN = false>
 __device__ __forceinline__ float residual_row(const MixedState &m, const double *__restrict__ r,
                                               const double *__restrict__ x, int s, int k, int i) {
   constexpr int NB2 = NB * NB;
@@ -784,38 +786,41 @@ __device__ __forceinline__ float residual_row(const MixedState &m, const double 
   const double ri = r[off + i];
   double acc = ri;
   float w = abs_f32_approx(ri);
-#pragma unroll
-  for (int j = 0; j < NB; ++j) {
-    const double kij = j <= i ? Dk[i * NB + j] : Dk[j * NB + i];
-    const double xj = xk[j];
+  auto term = [&](double kij, double xj) {
     acc = fma(-kij, xj, acc);
     w = fmaf(abs_f32_approx(kij), abs_f32_approx(xj), w);
+  };
+  auto block = [&](auto kij, const double *xv) {
+    if constexpr (LEAN && NB > 32) {
+#pragma unroll 8
+      for (int j = 0; j < NB; ++j) term(kij(j), xv[j]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < NB; ++j) term(kij(j), xv[j]);
+    }
+  };
+  if constexpr (LEAN) {   // along row i to the diagonal, then down column i
+    const double *d = Dk + i * NB;
+#pragma unroll
+    for (int j = 0; j < NB; ++j) {
+      term(*d, xk[j]);
+      d += j < i ? 1 : NB;
+    }
+  } else {
+    block([&](int j) { return j <= i ? Dk[i * NB + j] : Dk[j * NB + i]; }, xk);
   }
   if (k > 0) {   // block (k, k-1) = E_k (1-based stage k+1)
     const double *Ek = m.E + ((size_t)s * (N - 1) + (k - 1)) * NB2 + i * NB;
-    const double *xp = xk - NB;
-#pragma unroll
-    for (int j = 0; j < NB; ++j) {
-      acc = fma(-Ek[j], xp[j], acc);
-      w = fmaf(abs_f32_approx(Ek[j]), abs_f32_approx(xp[j]), w);
-    }
+    block([&](int j) { return Ek[j]; }, xk - NB);
   }
   if (k + 1 < N) {   // block (k, k+1) = E_{k+1}^T
     const double *Ek = m.E + ((size_t)s * (N - 1) + k) * NB2 + i;
-    const double *xn = xk + NB;
-#pragma unroll
-    for (int j = 0; j < NB; ++j) {
-      acc = fma(-Ek[j * NB], xn[j], acc);
-      w = fmaf(abs_f32_approx(Ek[j * NB]), abs_f32_approx(xn[j]), w);
-    }
+    block([&](int j) { return Ek[j * NB]; }, xk + NB);
   }
   if (k == 0) {   // block (1, root) = C_s^T
     const double *Cs = m.C + (size_t)s * nr * NB + i;
     const double *x0 = x + n0;
-    for (int j = 0; j < nr; ++j) {
-      acc = fma(-Cs[j * NB], x0[j], acc);
-      w = fmaf(abs_f32_approx(Cs[j * NB]), abs_f32_approx(x0[j]), w);
-    }
+    for (int j = 0; j < nr; ++j) term(Cs[j * NB], x0[j]);
   }
   m.rho[off + i] = acc;
   return omega_of(acc, w);
