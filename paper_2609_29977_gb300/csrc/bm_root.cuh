@@ -90,12 +90,67 @@ __device__ __forceinline__ void root_chol_store(double *sR, int nr, double *LR, 
   cta_store_lower(LR, sR, nr);
 }
 
-// The whole root step by one CTA: every entry (warps in turn), then the
-// Cholesky. sm: nr * nr + nr doubles of shared memory.
+// Whether root_reduce_chol takes 32 entries at a time (nr >= 6), and the
+// doubles of shared memory that it needs.
+__host__ __device__ constexpr bool root_by_columns(int nr) { return nr * (nr + 1) / 2 > 16; }
+__host__ __device__ constexpr int root_reduce_doubles(int nr) {
+  return root_by_columns(nr) && nr * nr + nr < 32 * 33 ? 32 * 33 : nr * nr + nr;
+}
+
+// The whole root step by one CTA (a multiple of four, at most eight warps):
+// every entry, then the Cholesky. Few entries: a warp per entry. More: one SM
+// reads all of U here, so the lanes of a warp read neighbouring entries: warp w adds up the partial sums p_l of
+// l = 4 w..4 w + 3 (and every 4 nw further on) for 32 entries at a time, sixteen loads in
+// flight, and the 32 partial sums of an entry are then combined by a warp, all in
+// the order of root_sum_warp. (With a warp per entry each load fetches 32
+// sectors for 8 bytes of each: factor of S = 512, N = 6, nb = 24, nr = 24 521 us,
+// 407 this way; nb = 16, nr = 6 113 and 105; nb = 4, nr = 4 31 and 35.)
+// sm: root_reduce_doubles(nr).
 __device__ __forceinline__ void root_reduce_chol(const double *U, const double *R, int S, int nr, double *Rt,
                                                  double *LR, Status *status, double *sm) {
-  const int ne = nr * (nr + 1) / 2, nw = blockDim.x >> 5;
-  for (int e = threadIdx.x >> 5; e < ne; e += nw) root_entry(U, R, S, nr, e, Rt);
+  const int ne = nr * (nr + 1) / 2, nw = blockDim.x >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const size_t stride = (size_t)nr * nr;
+  if (!root_by_columns(nr))
+    for (int e = w; e < ne; e += nw) root_entry(U, R, S, nr, e, Rt);
+  for (int e0 = 0; root_by_columns(nr) && e0 < ne; e0 += 32) {
+    int i, j;
+    tri_ij(e0 + lane < ne ? e0 + lane : ne - 1, i, j);
+    const double *Ue = U + i * nr + j;
+    for (int g = 4 * w; g < 32; g += 4 * nw) {
+      double acc[4] = {0.0, 0.0, 0.0, 0.0};
+      int s = g;
+      for (; s + 99 < S; s += 128) {
+        double v[4][4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) v[k][u] = __ldcg(Ue + (size_t)(s + 32 * k + u) * stride);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) acc[u] += v[k][u];
+      }
+      for (; s < S; s += 32)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (s + u < S) acc[u] += __ldcg(Ue + (size_t)(s + u) * stride);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) sm[(g + u) * 33 + lane] = acc[u];
+    }
+    __syncthreads();
+    for (int q = w; q < 32 && e0 + q < ne; q += nw) {
+      double acc = sm[lane * 33 + q];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (lane == 0) {
+        tri_ij(e0 + q, i, j);
+        const double val = R[i * nr + j] - acc;
+        Rt[i * nr + j] = val;
+        Rt[j * nr + i] = val;
+      }
+    }
+    __syncthreads();
+  }
   __threadfence_block();
   __syncthreads();
   for (int k = threadIdx.x; k < nr * nr; k += blockDim.x) sm[k] = Rt[k];

@@ -260,14 +260,37 @@ __global__ void __launch_bounds__(256) k_factor_level_team(TailView<T> v, int lv
 // Teams of the top kernel's CTA. For nb >= 24 two teams of four warps: with
 // four teams of two warps the factor of S = 512, N = 128, nb = 24 takes 3151
 // instead of 3122 us, and four of four spill (128 registers).
-template <typename T, int NB>
+template <int NB>
 constexpr int top_teams() {
   return NB <= 16 ? 4 : 2;
 }
+// The bound of its threads. (Below nb = 16 the plain operations need 60
+// registers with a bound of 512, up to 72 and spilling with their own.)
+template <int NB, int TEAM>
+constexpr int top_bound() {
+  return NB <= 12 ? 512 : TEAM * top_teams<NB>();
+}
+// Two teams of nb = 24 or 32 take 218 or 255 registers, one CTA per SM. With
+// more tails than SMs two CTAs at 128 registers, spilling, are faster
+// (MINB = 2), nb = 48 then has one team, and nb = 16 (116 registers, two CTAs of
+// four teams) two teams from 305 tails on. Factor, us, one CTA of two teams (nb = 16
+// two of four) -> this rule, nr = nb / 3: nb = 16, S = 512, N = 6 142 -> 105; nb = 24, S = 153, N = 6
+// 207 -> 150, S = 512, N = 6 402 -> 300, N = 64 1718 -> 1680; nb = 32, S = 304, N = 8
+// 455 -> 365; nb = 48, S = 153, N = 6 840 -> 618, S = 2000, N = 6 6472 -> 5311 (the
+// root step by columns, bm_root.cuh, included). At most 152 tails, capped: nb = 24,
+// S = 152, N = 8 144 -> 152, nb = 32 221 -> 240.
+template <int NB>
+constexpr bool top_capped() {
+  return NB == 24 || NB == 32;
+}
+template <int NB>
+int top_teams_for(int S) {
+  return NB == 48 && S > 152 ? 1 : NB == 16 && S > 304 ? 2 : top_teams<NB>();
+}
 
 // Top levels lvl0..Lc-1 and x_1 of one tail per CTA.
-template <typename T, int NB, int TEAM>
-__global__ void __launch_bounds__(TEAM * top_teams<T, NB>()) k_factor_top(TailView<T> v, int lvl0) {
+template <typename T, int NB, int TEAM, int MINB>
+__global__ void __launch_bounds__(top_bound<NB, TEAM>(), MINB) k_factor_top(TailView<T> v, int lvl0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *smem = (T *)smem_raw;
   const Team<TEAM> tm;
@@ -341,11 +364,13 @@ template <typename T, int NB, int TEAM>
 void launch_top(const TailView<T> &v, int lvl0, cudaStream_t st) {
   const size_t per = TeamSmem<T, NB>::bytes;
   const size_t x1b = x1_bytes<T, NB>(v.nr);
-  constexpr int tpc = top_teams<T, NB>();
+  const int tpc = top_teams_for<NB>(v.S);
   size_t smem = per * tpc > x1b ? per * tpc : x1b;
-  const size_t rootb = ((size_t)v.nr * v.nr + v.nr) * sizeof(double);
+  const size_t rootb = (size_t)root_reduce_doubles(v.nr) * sizeof(double);
   if (v.LR && rootb > smem) smem = rootb;
-  launch_pdl(k_factor_top<T, NB, TEAM>, (unsigned)v.S, TEAM * tpc, smem, st, v, lvl0);
+  constexpr int CAP = top_capped<NB>() ? 2 : 0;
+  launch_pdl(v.S > 152 ? k_factor_top<T, NB, TEAM, CAP> : k_factor_top<T, NB, TEAM, 0>, (unsigned)v.S, TEAM * tpc, smem,
+             st, v, lvl0);
 }
 
 template <typename T, int NB, int TEAM>
@@ -353,8 +378,11 @@ cudaError_t prepare_one() {
   cudaError_t e = cudaFuncSetAttribute(k_factor_level_team<T, NB, TEAM>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024);
   if constexpr (TEAM == team_top(NB)) {
+    constexpr int CAP = top_capped<NB>() ? 2 : 0;
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_factor_top<T, NB, TEAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024);
+    e = cudaFuncSetAttribute(k_factor_top<T, NB, TEAM, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_factor_top<T, NB, TEAM, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024);
   }
   return e;
 }

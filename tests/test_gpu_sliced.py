@@ -265,3 +265,29 @@ def test_decoupled_variable_with_a_subnormal_pivot(nb, col):
     _check_backward_error(d, fac, 1, 2.0 ** -53)
     assert fac["Ld"][s, k, col, col] == 2.0 ** -515
     assert x[((s * N + k) * nb) + col % nb] == 3.0
+
+
+@pytest.mark.parametrize("S,N,nb,nr", [(153, 3, 24, 5), (153, 6, 32, 6), (153, 3, 48, 16), (305, 5, 16, 7),
+                                       (305, 2, 12, 12), (161, 2, 24, 24)])
+def test_top_levels_of_many_tails_give_the_same_factor(S, N, nb, nr):
+    """The top kernel's forms for more tails than SMs, and the root's sums a
+    warp per entry or 32 entries at a time, against the same tails alone; the
+    root against the sum of their U in 64 bits."""
+    bm = _bm()
+    d = _gen(S, N, nb, nr)
+    _, fac, info = _run(d, flags=bm.BM_FLAG_NO_TUNE)
+    assert info["status"] == 0
+    keep = torch.tensor([0, 1, S - 2, S - 1])
+    few = dict(d, S=4, **{k: d[k][keep].contiguous() for k in ("D", "E", "C")})
+    few["r"] = torch.ones(4 * N * nb + nr, dtype=torch.float64)
+    _, ref, _ = _run(few, flags=bm.BM_FLAG_NO_TUNE)
+    for k in ("Ld", "Ll", "Lr", "F"):
+        assert np.array_equal(fac[k][keep.numpy()], ref[k]), k
+    F = fac["F"].astype(np.longdouble).reshape(S, nr, nb)
+    U = np.einsum("sik,sjk->ij", F, F)
+    R = np.tril(d["R"].numpy())
+    R = R + np.tril(R, -1).T
+    L = np.tril(fac["LR"]).astype(np.longdouble)
+    # S nb-term sums and nr terms of the Cholesky, each rounded
+    g = np.sqrt(np.diag(R).astype(np.longdouble))
+    assert float((np.abs(R - U - L @ L.T) / np.outer(g, g)).max()) <= (S + nb + nr + 2) * 2.0 ** -53
