@@ -339,15 +339,17 @@ __global__ void k_solve_x1_fwd(F64View v, const double *__restrict__ r) {
   }
 }
 
-// Root: r~_0 = r_0 - sum_i t_i (one warp per component, in the order of
-// root_sum_warp), then L_R L_R^T x_0 = r~_0 by one warp, a row per lane (and
-// row + 32 for nr > 32), and x_0. One CTA: with one per component and an
-// election of the last, block-wide sums and substitutions took 7 to 12 us
-// (nr = 2 to 16) of a chain whose arithmetic takes one to three
-// (S = 4, N = 16, nb = 4: factor and solve 56.2 -> 53.9 us).
+// Root: r~_0 = r_0 - sum_i t_i, then L_R L_R^T x_0 = r~_0 by one warp, a row
+// per lane (and row + 32 for nr > 32), and x_0. One CTA: with one per component
+// and an election of the last, block-wide sums and substitutions took 7 to 12 us
+// (nr = 2 to 16) of a chain whose arithmetic takes one to three. The threads
+// read tb contiguously: thread t adds component t mod nr over the tails
+// t / nr + k G, G = blockDim / nr, and a warp adds a component's G partial sums.
+// (A warp per component over all tails was latency and sectors of 8 bytes:
+// solve of S = 2000, N = 6, us: nb = 4, nr = 2 68 -> 62, nb = nr = 24 253 -> 238.)
 __global__ void __launch_bounds__(512) k_solve_root(F64View v, const double *__restrict__ r,
                                                     double *__restrict__ x) {
-  __shared__ double sL[64 * 65], sz[64], sInv[64];
+  __shared__ double sL[64 * 65], sz[64], sInv[64], part[512];
   const int nr = v.nr, S = v.S, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const size_t n0 = (size_t)S * v.N * v.nb;
   pdl_wait();
@@ -356,10 +358,24 @@ __global__ void __launch_bounds__(512) k_solve_root(F64View v, const double *__r
     sL[i * 65 + j] = v.LR[e];
     if (i == j) sInv[i] = 1.0 / v.LR[e];
   }
+  const int G = blockDim.x / nr, n = S * nr, step = G * nr;
+  double sum = 0.0;
+  if ((int)threadIdx.x < step) {
+    int e = threadIdx.x;
+    for (; e + 7 * step < n; e += 8 * step) {
+      double t[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) t[u] = __ldcg(v.tb + e + u * step);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) sum += t[u];
+    }
+    for (; e < n; e += step) sum += __ldcg(v.tb + e);
+  }
+  part[threadIdx.x] = sum;
+  __syncthreads();
   for (int c = warp; c < nr; c += blockDim.x >> 5) {
     double acc = 0.0;
-#pragma unroll 4
-    for (int s = lane; s < S; s += 32) acc += __ldcg(v.tb + (size_t)s * nr + c);
+    for (int g = lane; g < G; g += 32) acc += part[g * nr + c];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) sz[c] = r[n0 + c] - acc;
@@ -576,7 +592,10 @@ void f64_launch_export_ld(const F64View &v, double *Ld, cudaStream_t st) {
 }
 
 void f64_launch_solve_root(const F64View &v, const double *r, double *x, cudaStream_t st) {
-  launch_pdl(k_solve_root, 1u, 32u * (v.nr < 16 ? v.nr : 16), 0, st, v, r, x);
+  // a warp per component (16 at most), more while the sums have a term for each thread
+  const int comp = 32 * (v.nr < 16 ? v.nr : 16), terms = (v.S * v.nr + 31) / 32 * 32;
+  const int T = terms > 512 ? 512 : terms > comp ? terms : comp;
+  launch_pdl(k_solve_root, 1u, (unsigned)T, 0, st, v, r, x);
 }
 
 void f64_launch_solve(const F64View &v, const double *r, double *x, cudaStream_t st) {

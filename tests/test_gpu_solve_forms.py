@@ -68,6 +68,18 @@ def test_substitutions_and_residuals_give_the_batched_forms_bits(S, N, nb, tmp_p
     assert torch.equal(x, xb)
 
 
+# the root's sums: fewer tails than threads per component and more, components
+# that do and do not divide the threads
+@pytest.mark.parametrize("S,nr", [(1, 1), (1, 64), (5, 33), (7, 64), (130, 3), (513, 1), (600, 7), (90, 48)])
+def test_root_solve_over_sizes(S, nr):
+    import paper_2609_29977_gb300 as bm
+    from oracle import natural
+    w = bmgen.Workload("f", S, 2, 6, nr, workload_id=96, barrier=(-2.0, 2.0), shared_A=True)
+    d = bmgen.generate(w, seed=12)
+    x = _solve(bm, {k: (v.cuda() if isinstance(v, torch.Tensor) else v) for k, v in d.items()}, S).cpu().numpy()
+    assert natural.residual(d["D"], d["E"], d["C"], d["R"], x, d["r"])["eta"] <= 1e-12
+
+
 # five CTAs per SM where that saves a wave, four beside it
 @pytest.mark.parametrize("S,N,nb", [(608, 3, 4), (609, 3, 4), (760, 9, 6), (761, 2, 12), (700, 5, 24), (1217, 2, 6)])
 def test_substitutions_with_more_ctas_give_the_batched_forms_bits(S, N, nb, tmp_path, monkeypatch):
