@@ -569,22 +569,18 @@ __device__ __forceinline__ bool last_cta(unsigned *ticket, unsigned n) {
   return last != 0;
 }
 
-// The correction of a row, z, into y, x (xo before) and the planes of x.
-__device__ __forceinline__ void bwd_store(const MixedState &m, double *x, int iter, size_t row, float z, double xo,
-                                          bool xmode, const float *sdh, const float *sdl) {
+// With refined coupling columns the correction of row i is d_i = z - X_i d_0,
+// the product summed by Dot2 (h + l).
+__device__ __forceinline__ double coupled_correction(float z, float h, float l) {
+  float dh, e;
+  ff::two_sum(z, -h, dh, e);
+  return ff::to_double(dh, __fsub_rn(e, l));
+}
+
+// The correction of a row, z (dz in full), into y, x (xo before) and the planes of x.
+__device__ __forceinline__ void bwd_store(const MixedState &m, double *x, int iter, size_t row, float z, double dz,
+                                          double xo) {
   m.y[row] = z;
-  double dz;
-  if (xmode) {
-    // d_i = z - X_i d_0 on this row, the product summed by Dot2
-    const float *xr = m.Xc + row * m.ldc;
-    float h = 0.0f, l = 0.0f;
-    for (int c = 0; c < m.nr; ++c) ff::dot2_step_split(h, l, sdh[c], sdl[c], __ldcg(xr + c));
-    float dh, e;
-    ff::two_sum(z, -h, dh, e);
-    dz = ff::to_double(dh, __fsub_rn(e, l));
-  } else {
-    dz = f2d_exact(z);
-  }
   const double xv = iter == 0 ? dz : xo + dz;
   x[row] = xv;
   if (m.ffres) {
@@ -594,6 +590,38 @@ __device__ __forceinline__ void bwd_store(const MixedState &m, double *x, int it
     m.xl[row] = l;
     if (ff::out_of_range(xv)) m.status->ffbad = 1;
   }
+}
+__device__ __forceinline__ void bwd_store(const MixedState &m, double *x, int iter, size_t row, float z, double xo,
+                                          bool xmode, const float *sdh, const float *sdl) {
+  double dz;
+  if (xmode) {
+    const float *xr = m.Xc + row * m.ldc;
+    float h = 0.0f, l = 0.0f;
+    for (int c = 0; c < m.nr; ++c) ff::dot2_step_split(h, l, sdh[c], sdl[c], __ldcg(xr + c));
+    dz = coupled_correction(z, h, l);
+  } else {
+    dz = f2d_exact(z);
+  }
+  bwd_store(m, x, iter, row, z, dz, xo);
+}
+// Two rows of a lane with refined coupling columns (the second only where two
+// is set), their Dot2 chains side by side: one after the other they are a
+// chain twice as long as that of the two-warp teams that the pair form
+// replaced. Solve, S = 64, N = 60, nb = 48, us, teams; one after the other; this
+// way: 517, 559, 542; with FP64 residuals 566, 654, 590 (the residual's own kernel
+// included).
+__device__ __forceinline__ void bwd_store_coupled(const MixedState &m, double *x, int iter, size_t row0, size_t row1,
+                                                  bool two, float z0, float z1, double x0, double x1,
+                                                  const float *sdh, const float *sdl) {
+  const float *r0 = m.Xc + row0 * m.ldc, *r1 = m.Xc + row1 * m.ldc;
+  float h0 = 0.0f, l0 = 0.0f, h1 = 0.0f, l1 = 0.0f;
+#pragma unroll 4
+  for (int c = 0; c < m.nr; ++c) {
+    ff::dot2_step_split(h0, l0, sdh[c], sdl[c], __ldcg(r0 + c));
+    ff::dot2_step_split(h1, l1, sdh[c], sdl[c], __ldcg(r1 + c));
+  }
+  bwd_store(m, x, iter, row0, z0, coupled_correction(z0, h0, l0), x0);
+  if (two) bwd_store(m, x, iter, row1, z1, coupled_correction(z1, h1, l1), x1);
 }
 
 template <int NB>
@@ -654,8 +682,12 @@ __device__ __forceinline__ void bwd_tail_pair(const MixedState &m, double *x, in
           if (i0 < j) z0 = fmaf(-buf[SubCfg<NB>::row(j) + i0], xj, z0);
         }
       }
-      bwd_store(m, x, iter, zoff + i0, z0, x0, xmode, sdh, sdl);
-      if (two) bwd_store(m, x, iter, zoff + i1, z1, x1, xmode, sdh, sdl);
+      if (xmode) {
+        bwd_store_coupled(m, x, iter, zoff + i0, zoff + i1, two, z0, z1, x0, x1, sdh, sdl);
+      } else {
+        bwd_store(m, x, iter, zoff + i0, z0, f2d_exact(z0), x0);
+        if (two) bwd_store(m, x, iter, zoff + i1, z1, f2d_exact(z1), x1);
+      }
     }
     if (CS > 1)
       cluster_sync();
