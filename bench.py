@@ -55,6 +55,14 @@ def _peaks():
     return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "sm_max_mhz": 2070.0}, "fallback"
 
 
+def sliced_products(nb):
+    """Whether the FP64 factor of this block size forms its products as exact
+    digit products on the tensor cores (csrc/bm_sliced.cuh: the compiled
+    sizes from 16 on that are multiples of 8); every other size runs on the
+    FP64 ALU."""
+    return nb in (16, 24, 32, 48)
+
+
 def fp64_peak_gflops(sm_mhz=None):
     """FP64 ALU peak of the GPU: 152 SMs x 2 FMA lanes per clock (one 32-lane
     warp instruction per 64 cycles on each of the 4 SM sub-partitions,
@@ -835,10 +843,11 @@ def run_gpu(args):
                 "peak_source": peak_src,
                 "achieved_basis": "method flops of one factor (%.4g) / mean factor time over the timed "
                                   "steps (CUDA events on the launching stream)" % fl["factor"]}
-    if args.precision == "fp64" and w.nb >= 16:
-        # the products of blocks from 16 on run as exact digit products on the
-        # tensor cores, so the FP64 ALU's rate bounds nothing any more: the
-        # floor is the bytes
+    if args.precision == "fp64" and sliced_products(w.nb):
+        # the products run as exact digit products on the tensor cores, so the
+        # method's flops have no bound in the FP64 ALU's rate (Cholesky, panel
+        # inverses, F and U still run there and have a floor of their own): the
+        # bytes are a lower bound of the time
         roofline = {"bound": "hbm", "achieved": factor_gbs, "peak": _peaks()[0]["hbm_gbs"], "unit": "GB/s",
                     "frac": factor_gbs / _peaks()[0]["hbm_gbs"], "peak_source": _peaks()[1],
                     "achieved_basis": "algorithmic bytes of one factor (%.4g) / mean factor time over the timed "

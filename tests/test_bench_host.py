@@ -102,3 +102,19 @@ def test_factor_kernel_names_match_the_launch_counts():
     assert core.launches_per_step(64, 64, 12, 4) - 3 == 4 + 1
     assert bench._factor_kernels(256, 48, "fp32ir").startswith("k_level_rows_w x6 + k_top_rows_w + k_pivot_spread")
     assert bench._factor_kernels(9, 5, "fp64") == "k_factor_level x4 + k_factor_x1 + k_factor_root"
+
+
+def test_fp64_roofline_is_by_bytes_where_the_sliced_kernels_run():
+    """The compiled block sizes of csrc/bm_internal.cuh under the rule of
+    bm_sliced.cuh (a multiple of 8 from 16 on); generic sizes above 16 run on
+    the FP64 ALU."""
+    import os
+    import re
+    csrc = os.path.join(os.path.dirname(os.path.abspath(bench.__file__)), "paper_2609_29977_gb300", "csrc")
+    with open(os.path.join(csrc, "bm_internal.cuh")) as f:
+        line = next(t for t in f if t.startswith("#define BM_TAIL_NB_LIST"))
+    compiled = {int(v) for v in re.findall(r"X\((\d+)\)", line)}
+    with open(os.path.join(csrc, "bm_sliced.cuh")) as f:
+        assert "NB % 8 == 0 && NB >= 16" in f.read()
+    for nb in range(2, 65):
+        assert bench.sliced_products(nb) == (nb in compiled and nb % 8 == 0 and nb >= 16), nb
