@@ -1,6 +1,6 @@
 // Dispatch of the tail factorization on the block size (Alg. 1, steps 1-3).
-// The kernels are defined in bm_tail_factor.cuh and instantiated in
-// bm_tail_inst_*.cu.
+// The kernels are defined in bm_tail_factor.cuh (FP64), bm_tail_rows.cuh and
+// bm_tail_wide.cuh (FP32) and instantiated in bm_tail_inst_*.cu.
 #include <mutex>
 
 #include "bm_tail_factor.cuh"
@@ -11,12 +11,9 @@ namespace tail {
 #define X(n)                                                                                               \
   extern template void launch_tail_nb<double, n>(const TailView<double> &, cudaStream_t, const TailSched *, \
                                                  cudaEvent_t *);                                           \
-  extern template void launch_tail_nb<float, n>(const TailView<float> &, cudaStream_t, const TailSched *,   \
-                                                cudaEvent_t *);                                            \
   extern template void launch_tail_range<double, n>(const TailView<double> &, cudaStream_t, const TailSched *, \
                                                     int, int, bool, cudaEvent_t *);                            \
-  extern template cudaError_t prepare_nb<double, n>();                              \
-  extern template cudaError_t prepare_nb<float, n>();
+  extern template cudaError_t prepare_nb<double, n>();
 BM_TAIL_NB_LIST(X)
 #undef X
 }  // namespace tail
@@ -48,9 +45,8 @@ cudaError_t tail_factor_prepare() {
   if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorUnknown;
   if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
   cudaError_t e = cudaSuccess;
-#define X(n)                                                   \
-  if (e == cudaSuccess) e = tail::prepare_nb<double, n>();     \
-  if (e == cudaSuccess) e = tail::prepare_nb<float, n>();
+#define X(n) \
+  if (e == cudaSuccess) e = tail::prepare_nb<double, n>();
   BM_TAIL_NB_LIST(X)
 #undef X
 #define X(n) \
@@ -63,29 +59,31 @@ cudaError_t tail_factor_prepare() {
 }
 
 // Tail levels and x_1 of the factor (the root step is launched separately).
-// FP32 tails use the register-row kernels (three-warp teams for nb = 48).
+// FP32 tails use the register-row kernels (three-warp teams for nb = 48), which
+// have no schedule.
 template <typename T>
 void tail_factor_launch(const TailView<T> &v, cudaStream_t st, const TailSched *sc, cudaEvent_t *ev) {
-  if (sizeof(T) == 4) {
+  if constexpr (sizeof(T) == 4) {
     switch (v.nb) {
-#define X(n)                                                                        \
-  case n:                                                                           \
-    rows::launch_tail_rows<float, n>(*reinterpret_cast<const TailView<float> *>(&v), st); \
-    return;
+#define X(n)                              \
+  case n:                                 \
+    rows::launch_tail_rows<float, n>(v, st); \
+    break;
       BM_ROWS_NB_LIST(X)
 #undef X
       case 48:
-        rows::launch_tail_w<48>(*reinterpret_cast<const TailView<float> *>(&v), st);
-        return;
+        rows::launch_tail_w<48>(v, st);
+        break;
     }
-  }
-  switch (v.nb) {
-#define X(n)                           \
-  case n:                              \
+  } else {
+    switch (v.nb) {
+#define X(n)                                   \
+  case n:                                      \
     tail::launch_tail_nb<T, n>(v, st, sc, ev); \
     break;
-    BM_TAIL_NB_LIST(X)
+      BM_TAIL_NB_LIST(X)
 #undef X
+    }
   }
 }
 template void tail_factor_launch<double>(const TailView<double> &, cudaStream_t, const TailSched *, cudaEvent_t *);

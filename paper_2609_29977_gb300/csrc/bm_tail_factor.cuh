@@ -1,7 +1,7 @@
-// Tail factorization with compile-time block sizes and per-level team sizes
-// (Alg. 1, steps 1-3), for the FP64 path (T = double) and the FP32 tails of
-// the mixed-precision path (T = float: the FP64 inputs are rounded to
-// nearest on load; the coupling solve and the local Schur update stay FP64).
+// FP64 tail factorization with compile-time block sizes and per-level team
+// sizes (Alg. 1, steps 1-3). Instantiated for T = double; the FP32 tails of the
+// mixed-precision path have kernels of their own (bm_tail_rows.cuh,
+// bm_tail_wide.cuh).
 //
 // Same level schedule as the generic kernels in bm_fp64.cu (odd-even levels
 // of Gamma_{N-1}, Sec. II), organised for GB300:
@@ -50,7 +50,7 @@ __device__ __forceinline__ void team_load_t(const Team<TEAM> &tm, T *__restrict_
 
 // The block operations of a task: on the FP64 path the sliced products and
 // the pivots' reciprocals of bm_sliced.cuh for nb >= 16, the plain ones of
-// bm_team.cuh for smaller blocks and for FP32. Whole factor, plain -> sliced:
+// bm_team.cuh for smaller blocks. Whole factor, plain -> sliced:
 // S = 512, N = 128, nb = 24: 6216 -> 3122 us; S = 100, N = 160, nb = 16:
 // 807 -> 438; S = N = 64, nb = 32: 1525 -> 687, nb = 48: 4695 -> 1831. The
 // line lies below nb = 16: a product of 12 columns is padded to 16 and needs

@@ -1,14 +1,7 @@
-// Explicit instantiations of the tail factorization kernels (float, nb in [12, 16]).
-#include "bm_tail_factor.cuh"
+// Explicit instantiations of the FP32 tail kernels (nb in [12, 16]).
 #include "bm_tail_rows.cuh"
 
 namespace bm {
-namespace tail {
-template void launch_tail_nb<float, 12>(const TailView<float> &, cudaStream_t, const TailSched *, cudaEvent_t *);
-template cudaError_t prepare_nb<float, 12>();
-template void launch_tail_nb<float, 16>(const TailView<float> &, cudaStream_t, const TailSched *, cudaEvent_t *);
-template cudaError_t prepare_nb<float, 16>();
-}  // namespace tail
 template void rows::launch_tail_rows<float, 12>(const TailView<float> &, cudaStream_t);
 template cudaError_t rows::prepare_rows<float, 12>();
 template void rows::launch_tail_rows<float, 16>(const TailView<float> &, cudaStream_t);
