@@ -377,6 +377,7 @@ struct bm_batch_s {
   BTail *d_tails = nullptr;
   unsigned long long *d_heads = nullptr;
   int ncls = 0, ntails = 0, max_refine = 10;
+  int large_tails = 0;   // tails with at least half of the largest one's work
   double tol = 1e-10;
   int smem_per_team_max = 0, min_team_width = 32;
   std::vector<int> cls_nb, cls_team_bytes;
@@ -459,7 +460,7 @@ static void launch_factor(bm_batch_s *h, const double *const *D, const double *c
 static void launch_solve(bm_batch_s *h, const double *const *r, double *const *x, cudaStream_t st) {
   batch_launch_reset(h->d_inst, h->count, st);
   for (int it = 0; it <= h->max_refine; ++it)
-    batch_launch_solve_iteration(h->d_inst, h->d_tails, h->ntails, r, x, it, h->max_refine, h->tol, st);
+    batch_launch_solve_iteration(h->d_inst, h->d_tails, h->ntails, h->large_tails, r, x, it, h->max_refine, h->tol, st);
 }
 
 extern "C" bm_status bm_batch_analyze(const bm_desc *descs, int count, void *stream, bm_batch *out) {
@@ -587,6 +588,8 @@ extern "C" bm_status bm_batch_analyze(const bm_desc *descs, int count, void *str
   auto work = [&](const BTail &t) { return (long)descs[t.inst].N * descs[t.inst].nb * descs[t.inst].nb; };
   std::stable_sort(tails.begin(), tails.end(), [&](const BTail &a, const BTail &b) { return work(a) > work(b); });
   h->ntails = (int)tails.size();
+  h->large_tails = 0;
+  for (const BTail &t : tails) h->large_tails += 2 * work(t) >= work(tails[0]);
   bool ok = cudaMalloc(&h->d_inst, count * sizeof(BInst)) == cudaSuccess &&
             cudaMalloc(&h->d_cls, cls.size() * sizeof(BClass)) == cudaSuccess &&
             cudaMalloc(&h->d_segs, segs.size() * sizeof(BSeg)) == cudaSuccess &&

@@ -33,8 +33,9 @@ struct BTail {
 // {6, 12, 24, 48}; 4 is kept for small test systems).
 #define BM_BATCH_NB_LIST(X) X(4) X(6) X(12) X(24) X(48)
 
-void batch_launch_solve_iteration(const BInst *inst, const BTail *tails, int ntails, const double *const *r,
-                                  double *const *x, int iter, int max_iter, double tol, cudaStream_t st);
+void batch_launch_solve_iteration(const BInst *inst, const BTail *tails, int ntails, int large,
+                                  const double *const *r, double *const *x, int iter, int max_iter, double tol,
+                                  cudaStream_t st);
 void batch_launch_reset(BInst *inst, int ninst, cudaStream_t st);
 
 }  // namespace bm

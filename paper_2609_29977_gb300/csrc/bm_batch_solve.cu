@@ -66,10 +66,12 @@ __global__ void __launch_bounds__(256, 3) k_batch_bwd(const BInst *inst, const B
 }
 
 // MINB: CTAs per SM, three (80 registers), or four (64, some spilling) where
-// all tails then run in fewer waves. 16 systems of 30 tails, N = 60, solve, us,
+// the large tails (large: those with at least half of the largest one's
+// work) then run in fewer waves. 16 systems of 30 tails, N = 60, solve, us,
 // three -> four: nb = 6 478 -> 464, 12 740 -> 710, 24 1417 -> 1320, 48 3987 -> 3641;
 // with as many waves (8 systems of 100 tails, N = 100) 24 2809 -> 3015, 48
-// 7504 -> 8321.
+// 7504 -> 8321. By the number of all tails, a batch of 16 uneven systems took 5581 us
+// for factor and solve instead of 5344.
 inline bool four_ctas(long ctas) { return (ctas + 4 * 152 - 1) / (4 * 152) < (ctas + 3 * 152 - 1) / (3 * 152); }
 
 template <int MINB>
@@ -99,11 +101,12 @@ void batch_launch_reset(BInst *inst, int ninst, cudaStream_t st) {
   k_batch_reset<<<(ninst + 127) / 128, 128, 0, st>>>(inst, ninst);
 }
 
-void batch_launch_solve_iteration(const BInst *inst, const BTail *tails, int ntails, const double *const *r,
-                                  double *const *x, int iter, int max_iter, double tol, cudaStream_t st) {
+void batch_launch_solve_iteration(const BInst *inst, const BTail *tails, int ntails, int large,
+                                  const double *const *r, double *const *x, int iter, int max_iter, double tol,
+                                  cudaStream_t st) {
   launch_pdl(k_batch_fwd, (unsigned)ntails, 256, 0, st, inst, tails, r, x, iter);
   launch_pdl(k_batch_bwd, (unsigned)ntails, 256, 0, st, inst, tails, x, iter);
-  launch_pdl(four_ctas(ntails) ? k_batch_res<4> : k_batch_res<3>, (unsigned)ntails, 256, 0, st, inst, tails, r, x, iter,
+  launch_pdl(four_ctas(large) ? k_batch_res<4> : k_batch_res<3>, (unsigned)ntails, 256, 0, st, inst, tails, r, x, iter,
              max_iter, tol);
 }
 
