@@ -427,8 +427,9 @@ __device__ __forceinline__ int team_chol(const Team<TEAM> &tm, double *sA, doubl
 // exponent of 1/L_ll: y_l 2^-o_l (an offset of the exponents below) and
 // (L_pp^-1)_kl 2^o_l, both exact. Without it the backward error of the solve
 // grew with the spread of the units within a panel (emulated, 1e-16 at 2^0,
-// 1e-12 at 2^20, 2e-9 at 2^30). It costs 1.4% of factor and solve at S = 512,
-// N = 128, nb = 24 (3790 -> 3843 us), 0.9% at S = 100, N = 160, nb = 16 (603 -> 608).
+// 1e-12 at 2^20, 2e-9 at 2^30). With the offsets
+// read before the tiles it costs nothing at S = 512, N = 128, nb = 24 (factor and solve
+// 3727 us without it, 3684 with; read in every tile 3782).
 __device__ __forceinline__ int column_scale(double inv) { return 1023 - (__double2hiint(inv) >> 20); }   // (inv > 0)
 
 // Largest biased exponents E0, E1 of a panel's rows y0 (rows 0-7) and y1 (8-15), whose
@@ -497,11 +498,11 @@ __device__ __forceinline__ void team_invert_diagonal(const Team<TEAM> &tm, doubl
 // One panel of team_trsm_lt for 16 rows held in registers (x[h][g]: rows 0-7
 // and 8-15 of the tile): the columns before the panel act on it through the
 // lower triangle of L, then it is multiplied by the inverse of its diagonal
-// block, both scaled per column (column_scale). The accumulators of a product
+// block, both scaled per column (column_scale; o: this lane's offsets). The accumulators of a product
 // have the layout of the next one's operand, so nothing passes through shared
 // memory in between.
 template <int NB, int P>
-__device__ __forceinline__ void trsm_panel(double (&x)[2][NB / 8][2], const double *sA, const double *inv) {
+__device__ __forceinline__ void trsm_panel(double (&x)[2][NB / 8][2], const double *sA, const int (&o)[NB / 8]) {
   constexpr int c0 = 8 * P;
   const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
   if constexpr (P > 0) {
@@ -539,7 +540,7 @@ __device__ __forceinline__ void trsm_panel(double (&x)[2][NB / 8][2], const doub
   double b[1][2];
   load_rows<8>(b, sA + c0 * NB + c0, NB, gid, 8);
   const int Eb = row_exponent<1>(b);
-  const int o0 = column_scale(inv[c0 + 2 * tig]), o1 = column_scale(inv[c0 + 2 * tig + 1]);
+  const int o0 = o[P] >> 16, o1 = (int)(short)o[P];
   int E0, E1;
   row_exponents_scaled(x[0][P], x[1][P], o0, o1, E0, E1);
   unsigned a0[ND], a1[ND], bd[ND];
@@ -553,7 +554,7 @@ __device__ __forceinline__ void trsm_panel(double (&x)[2][NB / 8][2], const doub
 #pragma unroll
   for (int t = 0; t < 4; ++t)   // (entries of X: against sqrt(K_ii) > 2^-538 a subnormal one does not show)
     x[t >> 1][P][t & 1] = assemble<8>(c, t, t >> 1 ? E1 : E0, (t & 1) ? Eb1 : Eb0);
-  if constexpr (c0 + 8 < NB) trsm_panel<NB, P + 1>(x, sA, inv);
+  if constexpr (c0 + 8 < NB) trsm_panel<NB, P + 1>(x, sA, o);
 }
 
 // X (M x NB) := X L^{-T}, all of it sliced products, 16 rows per warp at a
@@ -565,12 +566,16 @@ __device__ __forceinline__ void team_trsm_lt(const Team<TEAM> &tm, double *X, in
   const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
   tm.sync();
   team_invert_diagonal<TEAM, NB>(tm, sA, inv);
+  int o[KG];   // the column offsets of this lane in every panel, two to a word
+#pragma unroll
+  for (int g = 0; g < KG; ++g)
+    o[g] = column_scale(inv[8 * g + 2 * tig]) << 16 | (column_scale(inv[8 * g + 2 * tig + 1]) & 0xffff);
 #pragma unroll 1
   for (int mt = tm.lane >> 5; mt * 16 < M; mt += TEAM / 32) {
     double x[2][KG][2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) load_rows<NB>(x[h], X, NB, mt * 16 + h * 8 + gid, M);
-    trsm_panel<NB, 0>(x, sA, inv);
+    trsm_panel<NB, 0>(x, sA, o);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int row = mt * 16 + h * 8 + gid;
