@@ -27,17 +27,18 @@
 //   * the seven sums are put together in 64-bit integers, at most two units
 //     short by truncation (2^-57 of X Y for K <= 24, 2^-56 above), and turned
 //     into a double by integer instructions, rounded to nearest, so a fill
-//     block needs no FP64 instruction and an update needs one subtraction per
-//     entry instead of nb (or 2 nb) FMAs.
+//     block needs one FP64 multiplication (up_scale) and an update one FMA per
+//     entry instead of nb (or 2 nb).
 //
 // Where each row carries one scale the loss stays within the backward error
 // of an FMA chain, nb 2^-53 sqrt(K_ii K_jj): rows of L and of X do (|x_i| <=
 // sqrt(K_ii), whatever the units of the variables), and the operands of the
 // panels' inverses are brought to it (column_scale). Measured componentwise
 // backward error of the solution, geometric mean over six generated systems
-// whose variables have like units, FMA chain -> sliced: 7.2e-16 -> 2.8e-16
-// (nb = 16), 6.8e-16 -> 2.7e-16 (24), 6.2e-16 -> 2.4e-16 (32), 5.7e-16 ->
-// 1.9e-16 (48). A row whose largest exponent is that of inf or NaN makes
+// whose variables have like units (before the columns were scaled, which moves
+// solutions of such systems by rounding only), FMA chain -> sliced: 7.2e-16 ->
+// 2.8e-16 (nb = 16), 6.8e-16 -> 2.7e-16 (24), 6.2e-16 -> 2.4e-16 (32), 5.7e-16
+// -> 1.9e-16 (48). A row whose largest exponent is that of inf or NaN makes
 // every product with it NaN, which a later pivot reports.
 //
 // What bounds the level kernels now (S = 128, N = 128, nb = 24, level 1, 242
