@@ -302,6 +302,14 @@ __global__ void __launch_bounds__(256) k_x_split(MixedState m, const double *__r
 
 // rho = r - K x with the refinement's arithmetic (bm_residual): m.rho is
 // the caller's array.
+// Sizes whose FP64 handles have a public residual of their own; the others
+// take the rows of the kernel for both (S = 512, N = 128, nb = 32 413 us, by a
+// kernel of its own 470).
+template <int NB>
+constexpr bool own_fp64_residual() {
+  return NB == 24 || NB == 48;
+}
+
 // FF as in k_mixed_residual. One kernel for both residuals took 165 registers
 // for nb = 48, one CTA per SM. S = 512, N = 128, us, that kernel -> this one:
 // float-float nb = 48 1000 -> 617, nb = 32 319 -> 313; FP64 nb = 48 1273 -> 1043,
@@ -311,7 +319,7 @@ __global__ void __launch_bounds__(256, !FF ? 0 : FFCfg<NB>::STAGED ? 3 : NB == 3
     k_residual_out(MixedState m, const double *__restrict__ r, const double *__restrict__ x) {
   extern __shared__ __align__(16) float sE[];
   const long nrow = (long)m.S * m.N * NB;
-  const bool ffr = FF && __ldcg(&m.status->ffbad) == 0;
+  const bool ffr = FF && m.ffres && __ldcg(&m.status->ffbad) == 0;
   if (ffr) {
     if constexpr (FF) residual_ff<NB>(m, r, x, sE);
   } else {
@@ -810,7 +818,7 @@ void mixed_launch_residual(MixedState *m, const double *r, const double *x, doub
   switch (m->nb) {
 #define X(n)                                                        \
   case n:                                                           \
-    if (c.ffres)                                                    \
+    if (c.ffres || !own_fp64_residual<n>())                         \
       k_residual_out<n, true><<<(unsigned)blocks, 256, FFCfg<n>::bytes, st>>>(c, r, x); \
     else                                                            \
       k_residual_out<n, false><<<(unsigned)blocks, 256, 0, st>>>(c, r, x); \
