@@ -300,8 +300,6 @@ __global__ void __launch_bounds__(256) k_x_split(MixedState m, const double *__r
   if (bad) m.status->ffbad = 1;
 }
 
-// rho = r - K x with the refinement's arithmetic (bm_residual): m.rho is
-// the caller's array.
 // Sizes whose FP64 handles have a public residual of their own; the others
 // take the rows of the kernel for both (S = 512, N = 128, nb = 32 413 us, by a
 // kernel of its own 470).
@@ -310,7 +308,9 @@ constexpr bool own_fp64_residual() {
   return NB == 24 || NB == 48;
 }
 
-// FF as in k_mixed_residual. One kernel for both residuals took 165 registers
+// rho = r - K x with the refinement's arithmetic (bm_residual): m.rho is
+// the caller's array. FF: float-float rows where the handle computes them, else
+// FP64 rows only (own_fp64_residual). Unbounded, the kernel for both took 165 registers
 // for nb = 48, one CTA per SM. S = 512, N = 128, us, that kernel -> this one:
 // float-float nb = 48 1000 -> 617, nb = 32 319 -> 313; FP64 nb = 48 1273 -> 1043,
 // nb = 24 255 -> 227.
